@@ -275,7 +275,15 @@ int rotgp_tune(rotgp_ctx* ctx, int axis, int lines_per_lane, int chunk, int ring
  *   for a cluster of 8 tiles of about 200 KB.
  * A new context uses ROTGP_SOLVER_THOMAS on every axis, except that complex
  * float axes with a halo above 16 points take ROTGP_SOLVER_HYBRID, and every
- * axis does when the halo exceeds 64 points. 
+ * axis does when the halo exceeds 64 points.
+ * While no form or shape has been asked for (rotgp_set_solver, rotgp_tune),
+ * 2D complex-float contexts whose tiles fit the SMs' shared memory (up to
+ * about 1100^2 points) and whose halo is at most 16 points run whole blocks
+ * of steps in one cooperative launch that keeps the state on chip (record
+ * "steps_2d" of rotgp_profile_read, one record per launch); results equal
+ * those of the sweeps up to float rounding and the same truncation bound.
+ * A wait between its tiles is bounded (about 2 s of device time,
+ * ROTGP_ETIMEOUT).
  * The y and z sweeps in stencil form, and the fused pass, stage their
  * tiles with TMA loads whose waits are bounded: a wait that runs out
  * (about 2 s) makes the next synchronising call return ROTGP_ETIMEOUT. */
@@ -293,8 +301,10 @@ int rotgp_set_solver(rotgp_ctx* ctx, int axis, int solver);
  * and the segment count of each stencil y/z sweep (as rotgp_tune).  Each candidate runs one warm-up step
  * and then twice `steps` imaginary-time steps from a copy of the current
  * state, timed with CUDA events on the context's stream (the faster repeat
- * counts); the state, its pending renormalisation and the step counter are
- * restored afterwards, and the fastest candidate stays selected.  *choice (if not NULL) receives it as a bit set: bit a =
+ * counts), and so does the on-chip 2D stepper where the context has one
+ * (selected, it shows as THOMAS on both axes); the state, its pending
+ * renormalisation and the step counter are restored afterwards, and the
+ * fastest candidate stays selected.  *choice (if not NULL) receives it as a bit set: bit a =
  * axis a in stencil form, bit 3 = fused x-y pass, bit 4 + a = axis a in the
  * exact partition solve (candidates include every supported combination
  * with it).  Synchronises the stream.

@@ -24,6 +24,7 @@
 
 #include "../../include/rotgp.h"
 #include "common.cuh"
+#include "resident.cuh"
 
 // A captured block of steps: valid for the instances' buffer parity at
 // capture time (the kernels' buffer pointers are part of the graph).
@@ -92,6 +93,17 @@ int run_set(rotgp_batch* b, const std::vector<int>& set, long long n, bool imag,
   return rc;
 }
 
+// Instances in the on-chip stepper (one cooperative launch over most of the
+// chip each, its CTAs waiting for one another) run one after another: instance
+// i waits for the one before it in the set.
+cudaError_t after_resident(rotgp_batch* b, int i, bool imag, int* before) {
+  if (!rotgp::ctx_resident(b->ctx[i], imag)) return cudaSuccess;
+  cudaError_t e = cudaSuccess;
+  if (*before >= 0) e = cudaStreamWaitEvent(b->streams[i], b->done[*before], 0);
+  *before = i;
+  return e;
+}
+
 int run_set_inner(rotgp_batch* b, const std::vector<int>& set, long long n, bool imag,
                   int mode) {
   cudaError_t e;
@@ -125,8 +137,10 @@ int run_set_inner(rotgp_batch* b, const std::vector<int>& set, long long n, bool
   if (mode != ROTGP_BATCH_GRAPH) {
     if ((e = cudaEventRecord(b->fork, b->stream)) != cudaSuccess)
       return bfail(b, ROTGP_ECUDA, "fork: %s", cudaGetErrorString(e));
+    int before = -1;  // the last instance in the on-chip stepper
     for (int i : set) {
-      if ((e = cudaStreamWaitEvent(b->streams[i], b->fork, 0)) != cudaSuccess)
+      if ((e = cudaStreamWaitEvent(b->streams[i], b->fork, 0)) != cudaSuccess ||
+          (e = after_resident(b, i, imag, &before)) != cudaSuccess)
         return bfail(b, ROTGP_ECUDA, "fork: %s", cudaGetErrorString(e));
       const int rc = imag ? rotgp_step_imag(b->ctx[i], n) : rotgp_step_real(b->ctx[i], n);
       if (rc) return bfail(b, rc, "instance %d: %s", i, rotgp_last_error(b->ctx[i]));
@@ -169,9 +183,11 @@ int run_set_inner(rotgp_batch* b, const std::vector<int>& set, long long n, bool
       return bfail(b, ROTGP_ECUDA, "begin capture: %s", cudaGetErrorString(e));
     int rc = ROTGP_OK;
     e = cudaEventRecord(b->fork, b->stream);
+    int before = -1;
     for (int i : set) {
       if (e != cudaSuccess || rc) break;
       e = cudaStreamWaitEvent(b->streams[i], b->fork, 0);
+      if (e == cudaSuccess) e = after_resident(b, i, imag, &before);
       if (e == cudaSuccess) {
         rc = imag ? rotgp_step_imag(b->ctx[i], n) : rotgp_step_real(b->ctx[i], n);
         if (rc) bfail(b, rc, "instance %d: %s", i, rotgp_last_error(b->ctx[i]));

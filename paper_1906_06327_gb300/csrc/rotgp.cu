@@ -17,6 +17,7 @@
 
 #include "../../include/rotgp.h"
 #include "common.cuh"
+#include "resident.cuh"
 #include "tma.cuh"
 
 using namespace rotgp;
@@ -30,12 +31,12 @@ constexpr int kMaxTable = 512;
 
 enum KernelId {
   K_SWEEP_X, K_SWEEP_Y, K_SWEEP_Z, K_OBS, K_VMOM, K_VCOUNT, K_NORM, K_INIT, K_IO, K_TABLES,
-  K_XY, K_COUNT
+  K_XY, K_RESIDENT, K_COUNT
 };
 const char* kKernelNames[K_COUNT] = {"sweep_x_h1",  "sweep_y",        "sweep_z",
                                      "observables", "vortex_moments", "vortex_count",
                                      "norm",        "init_analytic",  "pack_unpack",
-                                     "tables",      "xy_pass_h1"};
+                                     "tables",      "xy_pass_h1",     "steps_2d"};
 
 struct AxisPlan {
   int nlines = 0;       // lines with distinct coefficients (table rows)
@@ -61,7 +62,8 @@ struct AxisPlan {
   bool use_stencil = false;
   int sK = 0, sB = 0;
   int lsegs = 1;  // segments per line of the stencil line pass (y, z)
-  void* wtab[2] = {nullptr, nullptr};
+  void* wtab = nullptr;  // imaginary time only (real time never takes the stencil)
+  bool wtab_fresh = false;
   // exact partition-method solve (hybrid.cu): clusters of hcs CTAs, each a
   // tile of 16 lines x hpc positions, hlsub positions per thread
   bool hyb_ok = false;
@@ -116,6 +118,15 @@ struct rotgp_ctx {
   // [buffer][axis - 1][C = 8, 16]
   bool smaps_ok = false;
   CUtensorMap map_s1[2][2][2];
+  // on-chip 2D stepper (resident.cu): complex float, while the plan is the
+  // default one (no form or shape asked for); plans and tables per mode
+  bool user_plan = false;
+  bool res_ok[2] = {false, false};
+  res_plan rplan[2];
+  float2* rtab[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};  // [axis][mode]
+  float2* rsched[2] = {nullptr, nullptr};  // tables of kResSchedule steps, per axis
+  unsigned long long* xbuf = nullptr;      // two exchange planes,
+  res_sync* rsync = nullptr;               // ... the exchange words (and rtab) behind them
   double* partials = nullptr;
   size_t partial_doubles = 0;
   unsigned* counter = nullptr;
@@ -446,7 +457,7 @@ int plan_axes(rotgp_ctx* c) {
     // banded-inverse stencil: complex float, even N_x (TMA rows of 16-byte
     // multiples; the separate x-stencil kernel also wants N_x % 4 == 0)
     int K = 0, B = 0;
-    const bool sized = ap.wtab[0] != nullptr;  // tables already allocated
+    const bool sized = ap.wtab != nullptr;  // tables already allocated
     ap.stencil_ok = !c->fp64 && c->nx % 2 == 0 && plan_stencil(c, a, &K, &B);
     if (sized) {
       // keep the allocated size; a larger K or B than needed is only more exact
@@ -479,7 +490,7 @@ int plan_axes(rotgp_ctx* c) {
     c->fuse_ok = c->fuse_xy = false;
     return ROTGP_OK;
   }
-  if (!ax.wtab[0] && ax.stencil_ok && ay.stencil_ok) {
+  if (!ax.wtab && ax.stencil_ok && ay.stencil_ok) {
     const int K = std::max(ax.sK, ay.sK);
     ax.sK = ay.sK = K;
     c->fuse_ok = tile_k_built(K);
@@ -638,20 +649,97 @@ struct Timed {
   }
 };
 
+// The stencil weights of every axis that runs in stencil form (or in the
+// fused pass) now, where they do not match the physics yet.  Each weight row
+// is a set of short Thomas solves in double, some hundred times the work of
+// the Thomas tables, and most contexts never use them: they are built when a
+// form that reads them is selected (2D 512^2: 0.8 ms per axis, which every
+// step of an Omega schedule and every context creation paid before).
+int stencil_weights(rotgp_ctx* c) {
+  for (int a = 0; a < c->grid.dim; ++a) {
+    AxisPlan& ap = c->axis[a];
+    if (!ap.use_stencil || !ap.stencil_ok || !ap.wtab || ap.wtab_fresh) continue;
+    Timed t(c, K_TABLES);
+    const cudaError_t e = launch_stencil_tables(ap.wtab, ap.nlines, ap.sK, ap.sB,
+                                                2 * ap.sB + 2 * ap.sK + 8, ap.co[1], c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "table kernel");
+    ap.wtab_fresh = true;
+  }
+  return ROTGP_OK;
+}
+
 int build_tables(rotgp_ctx* c) {
   for (int a = 0; a < c->grid.dim; ++a) {
     AxisPlan& ap = c->axis[a];
+    ap.wtab_fresh = false;
     for (int mode = 0; mode < 2; ++mode) {
       ap.co[mode] = make_coef(a, mode, c->grid.h[a], c->phys.dt, c->phys.omega,
                               nlines_u0(c, a), nlines_du(c, a));
       Timed t(c, K_TABLES);
       cudaError_t e = launch_tables(c->fp64, ap.table[mode], ap.tableT[mode], ap.nlines, c->lt,
                                     ap.co[mode], c->stream);
-      if (e == cudaSuccess && ap.stencil_ok && ap.wtab[mode])
-        e = launch_stencil_tables(ap.wtab[mode], ap.nlines, ap.sK, ap.sB,
-                                  2 * ap.sB + 2 * ap.sK + 8, ap.co[mode], c->stream);
+      if (e == cudaSuccess && a < 2 && c->rtab[a][mode]) {
+        const res_omegas one{{1.0}};
+        e = launch_res_tables(c->rtab[a][mode], ap.nlines, c->lt, ap.co[mode], one, 1,
+                              c->stream);
+      }
       if (e != cudaSuccess) return cuda_fail(c, e, "table kernel");
     }
+  }
+  return stencil_weights(c);
+}
+
+// Does a step of this mode run in the on-chip stepper?  2D complex float
+// states whose tiles fit the shared memory and whose carries need a halo of
+// at most 16 points, unless a form or shape was asked for.
+bool resident(const rotgp_ctx* c, bool imag) {
+  return c->res_ok[imag ? 1 : 0] && !c->user_plan && c->chunk_ok &&
+         c->halo <= c->rplan[imag ? 1 : 0].H + 2;
+}
+
+// n steps in the on-chip stepper; tables: those of n steps in turn (a
+// schedule), or null for the context's own.
+int resident_steps(rotgp_ctx* c, long long n, bool imag, float2* const* tables) {
+  const int mode = imag ? 1 : 0;
+  res_args a{};
+  a.xbuf = c->xbuf;
+  a.xplane = 2 * (size_t)c->nx * c->ny;
+  a.tabx = tables ? tables[0] : c->rtab[0][mode];
+  a.taby = tables ? tables[1] : c->rtab[1][mode];
+  if (tables) {
+    a.step_x = (long long)kResPlanes * c->ny;
+    a.step_y = (long long)kResPlanes * c->nx;
+  }
+  a.nx = c->nx;
+  a.ny = c->ny;
+  a.plan = c->rplan[mode];
+  a.dt = (float)c->phys.dt;
+  a.g = (float)c->phys.g;
+  a.hgam2 = (float)(0.5 * c->phys.gamma * c->phys.gamma);
+  a.hnu2 = (float)(0.5 * c->phys.nu * c->phys.nu);
+  a.x0 = c->x0;
+  a.hx = c->grid.h[0];
+  a.y0 = c->y0;
+  a.hy = c->grid.h[1];
+  a.vol = c->vol;
+  a.scale = c->d_scale();
+  a.norm = c->d_norm();
+  a.flags = c->d_flags();
+  a.sync = c->rsync;
+  a.ex0 = (int)std::max(-60.0, std::min(60.0, std::floor(-std::log2(c->vol)) + 1.0));
+  // launches of at most 4096 steps (some 15 ms each)
+  for (long long s = 0; s < n; s += a.nsteps) {
+    a.nsteps = (int)std::min<long long>(4096, n - s);
+    a.in = static_cast<const float2*>(c->psi[c->cur]);
+    a.out = static_cast<float2*>(c->psi[1 - c->cur]);
+    cudaError_t e;
+    {
+      Timed t(c, K_RESIDENT);
+      e = launch_resident(imag, a, c->stream);
+    }
+    if (e != cudaSuccess) return cuda_fail(c, e, "on-chip stepper launch");
+    c->cur = 1 - c->cur;
+    c->steps += a.nsteps;
   }
   return ROTGP_OK;
 }
@@ -659,11 +747,10 @@ int build_tables(rotgp_ctx* c) {
 // --------------------------------------------------------------- one step
 tile_args make_tile_args(rotgp_ctx* c, bool imag) {
   tile_args t{};
-  const int mode = imag ? 1 : 0;
   t.out = c->psi[1 - c->cur];
-  t.wx = c->axis[0].wtab[mode];
-  t.wy = c->axis[1].wtab[mode];
-  t.wz = c->grid.dim == 3 ? c->axis[2].wtab[mode] : nullptr;
+  t.wx = c->axis[0].wtab;
+  t.wy = c->axis[1].wtab;
+  t.wz = c->grid.dim == 3 ? c->axis[2].wtab : nullptr;
   t.nx = c->nx;
   t.ny = c->ny;
   t.nz = c->nz;
@@ -741,7 +828,7 @@ int sweep(rotgp_ctx* c, int axis, bool imag, bool last) {
   a.scale_out = c->d_scale();
   a.norm_out = c->d_norm();
   a.flags = c->d_flags();
-  a.wtab = ap.wtab[mode];
+  a.wtab = ap.wtab;
   a.taps_k = ap.sK;
   a.brows = ap.sB;
   cudaError_t e;
@@ -831,6 +918,7 @@ int sweep(rotgp_ctx* c, int axis, bool imag, bool last) {
 int run_steps(rotgp_ctx* c, long long n, bool imag) {
   if (!c) return ROTGP_EINVAL;
   if (n < 0) return fail(c, ROTGP_EINVAL, "negative step count");
+  if (resident(c, imag)) return resident_steps(c, n, imag, nullptr);
   for (long long s = 0; s < n; ++s) {
     for (int a = 0; a < c->grid.dim; ++a) {
       int rc;
@@ -852,6 +940,28 @@ int run_steps(rotgp_ctx* c, long long n, bool imag) {
   return ROTGP_OK;
 }
 
+// The table space of a schedule of the on-chip stepper, allocated by the
+// first schedule (false: no space, or the stream is being captured, where
+// nothing may be allocated; such calls rebuild the tables step by step).
+bool schedule_tables(rotgp_ctx* c) {
+  if (c->rsched[1]) return true;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
+  for (int a = 0; a < 2; ++a) {
+    const size_t bytes = (size_t)kResSchedule * kResPlanes * c->axis[a].nlines * sizeof(float2);
+    if (cudaMalloc((void**)&c->rsched[a], bytes) != cudaSuccess) {
+      cudaGetLastError();
+      for (float2*& p : c->rsched) cudaFree(p), p = nullptr;
+      return false;
+    }
+    c->device_bytes += bytes;
+  }
+  return true;
+}
+
 int check_flags(rotgp_ctx* c) {
   int flags = 0;
   cudaError_t e = cudaMemcpyAsync(&flags, c->d_flags(), sizeof(int), cudaMemcpyDeviceToHost,
@@ -860,6 +970,12 @@ int check_flags(rotgp_ctx* c) {
   if (e != cudaSuccess) return cuda_fail(c, e, "synchronise");
   if (flags & 2) return fail(c, ROTGP_ECUDA, "a sweep kernel was launched with a shape it was not built for");
   if (flags & 4) return fail(c, ROTGP_ETIMEOUT, "a tile pass gave up waiting for its TMA load");
+  if (flags & 8) {
+    // no tag of the abandoned steps may be taken for one of a later launch
+    cudaMemsetAsync(c->rsync, 0, sizeof(res_sync), c->stream);
+    cudaMemsetAsync(c->xbuf, 0, 4 * (size_t)c->sites * sizeof(unsigned long long), c->stream);
+    return fail(c, ROTGP_ETIMEOUT, "a tile of the on-chip stepper gave up waiting for the others");
+  }
   if (flags & 1) return fail(c, ROTGP_ENONFINITE, "non-finite or zero norm in a reduction");
   return ROTGP_OK;
 }
@@ -877,8 +993,12 @@ void release(rotgp_ctx* c) {
   cudaFree(c->dR);
   for (auto& ap : c->axis) {
     for (void*& t : ap.table) cudaFree(t), t = nullptr;
-    for (void*& t : ap.wtab) cudaFree(t), t = nullptr;
+    for (void*& t : ap.tableT) cudaFree(t), t = nullptr;
+    cudaFree(ap.wtab);
+    ap.wtab = nullptr;
   }
+  for (float2*& p : c->rsched) cudaFree(p), p = nullptr;
+  cudaFree(c->xbuf);  // and the exchange words and weights behind the planes
   cudaFree(c->partials);
   cudaFree(c->counter);
   cudaFree(c->scalars);
@@ -937,6 +1057,7 @@ int encode_state_map(CUtensorMap* map, void* base, int nx, int ny, int nz, unsig
 int ctx_buffer(const rotgp_ctx* c) { return c->cur; }
 void ctx_set_buffer(rotgp_ctx* c, int cur) { c->cur = cur; }
 long long ctx_steps(const rotgp_ctx* c) { return c->steps; }
+bool ctx_resident(const rotgp_ctx* c, bool imag) { return resident(c, imag); }
 long long ctx_plan_version(const rotgp_ctx* c) { return c->plan_version; }
 void ctx_add_steps(rotgp_ctx* c, long long n) { c->steps += n; }
 void ctx_get_view(const rotgp_ctx* c, ctx_view* v) {
@@ -1108,7 +1229,7 @@ int rotgp_create(const rotgp_grid* grid, const rotgp_phys* phys, int precision, 
     AxisPlan& ap = c->axis[a];
     if (!ap.stencil_ok) continue;
     const size_t bytes = (size_t)ap.nlines * (2 * ap.sB + 1) * (2 * ap.sK + 1) * sizeof(cpx<float>);
-    for (int m = 0; m < 2 && !rc; ++m) rc = dev_alloc(c, &ap.wtab[m], bytes);
+    rc = dev_alloc(c, &ap.wtab, bytes);
   }
   if (!rc) {
     // the tile passes reduce the norm in their own blocks
@@ -1136,6 +1257,29 @@ int rotgp_create(const rotgp_grid* grid, const rotgp_phys* phys, int precision, 
     if (e == cudaSuccess) e = launch_set_scalar(c->d_scale(), 1.0, c->stream);
     if (e != cudaSuccess) rc = cuda_fail(c, e, "initialise buffers");
   }
+  if (!rc && grid->dim == 2 && !c->fp64 && c->chunk_ok && c->halo <= 16) {
+    // the on-chip stepper: plans, tables, exchange planes
+    for (int m = 0; m < 2; ++m)
+      c->res_ok[m] = res_make_plan(c->nx, c->ny, c->halo, m == 1, c->sm_count,
+                                   (size_t)c->smem_optin - 4096, &c->rplan[m]);
+    if (c->res_ok[0] || c->res_ok[1]) {
+      // one allocation: exchange planes, exchange words, the lines' weights
+      const size_t planes = 4 * (size_t)c->sites * sizeof(unsigned long long);
+      const size_t sync = (sizeof(res_sync) + 255) & ~(size_t)255;
+      const size_t wx = (size_t)kResPlanes * c->ny, wy = (size_t)kResPlanes * c->nx;
+      rc = dev_alloc(c, (void**)&c->xbuf, planes + sync + 2 * (wx + wy) * sizeof(float2));
+      if (!rc) {
+        c->rsync = reinterpret_cast<res_sync*>(reinterpret_cast<char*>(c->xbuf) + planes);
+        float2* w = reinterpret_cast<float2*>(reinterpret_cast<char*>(c->rsync) + sync);
+        for (int m = 0; m < 2; ++m) {
+          c->rtab[0][m] = w + m * (wx + wy);
+          c->rtab[1][m] = c->rtab[0][m] + wx;
+        }
+        e = cudaMemsetAsync(c->xbuf, 0, planes + sync, c->stream);
+        if (e != cudaSuccess) rc = cuda_fail(c, e, "initialise buffers");
+      }
+    }
+  }
   if (!rc) build_maps(c);
   if (!rc) lean_defaults(c);
   if (!rc) rc = build_tables(c);
@@ -1154,6 +1298,7 @@ int rotgp_create(const rotgp_grid* grid, const rotgp_phys* phys, int precision, 
   c->bytes_per_launch[K_SWEEP_Y] = 2.0 * state;
   c->bytes_per_launch[K_SWEEP_Z] = 2.0 * state;
   c->bytes_per_launch[K_XY] = 2.0 * state;
+  c->bytes_per_launch[K_RESIDENT] = 2.0 * state;
   c->bytes_per_launch[K_OBS] = 1.0 * state;
   *out = c;
   return ROTGP_OK;
@@ -1353,6 +1498,27 @@ int rotgp_step_schedule(rotgp_ctx* c, long long n, int imag, const double* omega
                   big);
   }
   const int mode = imag ? 1 : 0;
+  if (resident(c, imag != 0) && schedule_tables(c)) {
+    // tables of up to kResSchedule steps in one launch per axis, then those
+    // steps in one launch of the on-chip stepper
+    for (long long k = 0; k < n; k += kResSchedule) {
+      const int m = (int)std::min<long long>(kResSchedule, n - k);
+      res_omegas om{};
+      std::copy(omega + k, omega + k + m, om.v);
+      for (int a = 0; a < 2; ++a) {
+        const axis_coef co = make_coef(a, mode, c->grid.h[a], c->phys.dt, 1.0, nlines_u0(c, a),
+                                       nlines_du(c, a));
+        Timed t(c, K_TABLES);
+        const cudaError_t e = launch_res_tables(c->rsched[a], c->axis[a].nlines, c->lt, co, om, m,
+                                                c->stream);
+        if (e != cudaSuccess) return cuda_fail(c, e, "table kernel");
+      }
+      const int rc = resident_steps(c, m, imag != 0, c->rsched);
+      if (rc) return rc;
+    }
+    c->phys.omega = omega[n - 1];
+    return build_tables(c);
+  }
   for (long long k = 0; k < n; ++k) {
     if (omega[k] != c->phys.omega) {
       // the x and y tables of this mode (z lines carry no rotation term)
@@ -1364,13 +1530,12 @@ int rotgp_step_schedule(rotgp_ctx* c, long long n, int imag, const double* omega
         Timed t(c, K_TABLES);
         cudaError_t e = launch_tables(c->fp64, ap.table[mode], ap.tableT[mode], ap.nlines, c->lt,
                                       ap.co[mode], c->stream);
-        if (e == cudaSuccess && ap.stencil_ok && ap.wtab[mode])
-          e = launch_stencil_tables(ap.wtab[mode], ap.nlines, ap.sK, ap.sB,
-                                    2 * ap.sB + 2 * ap.sK + 8, ap.co[mode], c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "table kernel");
+        ap.wtab_fresh = false;
       }
     }
-    const int rc = run_steps(c, 1, imag != 0);
+    int rc = imag ? stencil_weights(c) : ROTGP_OK;
+    if (!rc) rc = run_steps(c, 1, imag != 0);
     if (rc) return rc;
   }
   // the other mode's tables follow the final Omega too
@@ -1511,6 +1676,7 @@ int rotgp_tune(rotgp_ctx* c, int axis, int lines_per_lane, int chunk, int ring,
       return fail(c, ROTGP_EINVAL, "segments must be 1..%d and leave >= 8 points each",
                   kMaxLineSegs);
     c->axis[axis].lsegs = segments;
+    c->user_plan = true;
     return ROTGP_OK;
   }
   if (axis < 0 || axis >= c->grid.dim) return fail(c, ROTGP_EINVAL, "axis out of range");
@@ -1542,6 +1708,7 @@ int rotgp_tune(rotgp_ctx* c, int axis, int lines_per_lane, int chunk, int ring,
     c->axis[axis] = keep;
     return rc;
   }
+  c->user_plan = true;
   return ROTGP_OK;
 }
 
@@ -1560,6 +1727,7 @@ int rotgp_set_solver(rotgp_ctx* c, int axis, int solver) {
     ap.use_hybrid = true;
     ap.use_stencil = false;
     if (axis <= 1) c->fuse_xy = false;
+    c->user_plan = true;
     return ROTGP_OK;
   }
   if (!c->chunk_ok)
@@ -1572,7 +1740,8 @@ int rotgp_set_solver(rotgp_ctx* c, int axis, int solver) {
     c->axis[0].use_stencil = c->axis[1].use_stencil = true;
     c->axis[0].use_hybrid = c->axis[1].use_hybrid = false;
     c->fuse_xy = true;
-    return ROTGP_OK;
+    c->user_plan = true;
+    return stencil_weights(c);
   }
   if (solver == ROTGP_SOLVER_STENCIL &&
       (!ap.stencil_ok || (axis == 0 && c->nx % 4 != 0 && !c->xpass_ok)))
@@ -1580,7 +1749,8 @@ int rotgp_set_solver(rotgp_ctx* c, int axis, int solver) {
   ap.use_stencil = solver == ROTGP_SOLVER_STENCIL;
   ap.use_hybrid = false;
   if (axis <= 1) c->fuse_xy = false;
-  return ROTGP_OK;
+  c->user_plan = true;
+  return stencil_weights(c);
 }
 
 int rotgp_autotune(rotgp_ctx* c, int steps, int* choice) {
@@ -1622,13 +1792,15 @@ int rotgp_autotune(rotgp_ctx* c, int steps, int* choice) {
       c->axis[a].use_stencil = ((m >> a) & 1) != 0;
       c->axis[a].use_hybrid = ((m >> (4 + a)) & 1) != 0;
     }
+    return stencil_weights(c);
   };
   // save the state, its pending scale and the counters
   const size_t state = (size_t)c->sites * c->elem;
   const int cur0 = c->cur;
   const long long steps0 = c->steps;
-  const bool prof0 = c->prof;
+  const bool prof0 = c->prof, plan0 = c->user_plan;
   c->prof = false;
+  c->user_plan = true;  // the sweep forms first
   double* saved_scale = reinterpret_cast<double*>(static_cast<char*>(c->staging) + state);
   cudaError_t e = cudaMemcpyAsync(c->staging, c->psi[cur0], state, cudaMemcpyDeviceToDevice,
                                   c->stream);
@@ -1667,7 +1839,7 @@ int rotgp_autotune(rotgp_ctx* c, int steps, int* choice) {
     return true;
   };
   for (size_t i = 0; i < cand.size() && e == cudaSuccess && !rc; ++i) {
-    apply(cand[i]);
+    if ((rc = apply(cand[i]))) break;
     float ms = 0;
     if (!time_current(&ms)) break;
     if (i == 0 || ms < best_ms) {
@@ -1675,7 +1847,7 @@ int rotgp_autotune(rotgp_ctx* c, int steps, int* choice) {
       best = cand[i];
     }
   }
-  apply(best);
+  if (!rc) rc = apply(best);
   // then the launch shapes of the Thomas sweeps (chunk, ring, segments: the
   // number of warps decides how many waves of resident warps a launch takes)
   for (int ax = 0; ax < dim && e == cudaSuccess && !rc; ++ax) {
@@ -1741,6 +1913,17 @@ int rotgp_autotune(rotgp_ctx* c, int steps, int* choice) {
     }
     ap.lsegs = best_s;
   }
+  // and the on-chip 2D stepper, which takes no form or shape
+  if (e == cudaSuccess && !rc) {
+    c->user_plan = false;
+    float ms = 0;
+    if (resident(c, true) && time_current(&ms) && ms < best_ms)
+      best = 0;
+    else
+      c->user_plan = true;
+    if (!c->user_plan && e == cudaSuccess && !rc) rc = apply(0);
+  }
+  if (e != cudaSuccess || rc) c->user_plan = plan0;
   for (cudaEvent_t x : ev)
     if (x) cudaEventDestroy(x);
   const cudaError_t er = restore();
