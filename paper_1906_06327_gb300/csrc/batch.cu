@@ -24,6 +24,7 @@
 
 #include "../../include/rotgp.h"
 #include "common.cuh"
+#include "observe.cuh"
 #include "resident.cuh"
 
 // A captured block of steps: valid for the instances' buffer parity at
@@ -78,6 +79,21 @@ void drop_graph(rotgp_batch* b) {
 
 int run_set_inner(rotgp_batch* b, const std::vector<int>& set, long long n, bool imag,
                   int mode);
+
+// The observables of the instances in `set`, all enqueued on their streams
+// before the first is waited for.
+int observe_set(rotgp_batch* b, const std::vector<int>& set, rotgp_obs* out) {
+  for (int i : set) {
+    const int rc = rotgp::ctx_observe(b->ctx[i]);
+    if (rc) return bfail(b, rc, "instance %d: %s", i, rotgp_last_error(b->ctx[i]));
+  }
+  int first = ROTGP_OK;
+  for (size_t k = 0; k < set.size(); ++k) {
+    const int rc = rotgp::ctx_observed(b->ctx[set[k]], &out[k]);
+    if (rc && !first) first = bfail(b, rc, "instance %d: %s", set[k], rotgp_last_error(b->ctx[set[k]]));
+  }
+  return first;
+}
 
 // Run n steps of the instances in `set` (mode: ROTGP_BATCH_*), ordered after
 // the caller's stream and before its next work.
@@ -330,12 +346,10 @@ int rotgp_batch_sync(rotgp_batch* b) {
 
 int rotgp_batch_observables(rotgp_batch* b, rotgp_obs* out) {
   if (!b || !out) return ROTGP_EINVAL;
-  int rc = rotgp_batch_sync(b);
-  for (size_t i = 0; i < b->ctx.size() && !rc; ++i) {
-    rc = rotgp_observables(b->ctx[i], &out[i]);
-    if (rc) bfail(b, rc, "instance %zu: %s", i, rotgp_last_error(b->ctx[i]));
-  }
-  return rc;
+  std::vector<int> all(b->ctx.size());
+  for (size_t i = 0; i < all.size(); ++i) all[i] = (int)i;
+  const int rc = rotgp_batch_sync(b);
+  return rc ? rc : observe_set(b, all, out);
 }
 
 int rotgp_batch_converge(rotgp_batch* b, double rel_tol, long long check_every,
@@ -362,10 +376,11 @@ int rotgp_batch_converge(rotgp_batch* b, double rel_tol, long long check_every,
     if (!rc) rc = rotgp_batch_sync(b);
     if (rc) return rc;
     done_steps += k;
-    for (int i : active) {
-      rotgp_obs o;
-      rc = rotgp_observables(b->ctx[i], &o);
-      if (rc) return bfail(b, rc, "instance %d: %s", i, rotgp_last_error(b->ctx[i]));
+    std::vector<rotgp_obs> obs(active.size());
+    if ((rc = observe_set(b, active, obs.data()))) return rc;
+    for (size_t k2 = 0; k2 < active.size(); ++k2) {
+      const int i = active[k2];
+      const rotgp_obs& o = obs[k2];
       steps_out[i] = done_steps;
       if (std::isfinite(mu[i]) && std::fabs(o.mu - mu[i]) <= rel_tol * std::fabs(o.mu) &&
           o.vortices == vort[i])

@@ -17,6 +17,7 @@
 
 #include "../../include/rotgp.h"
 #include "common.cuh"
+#include "observe.cuh"
 #include "resident.cuh"
 #include "tma.cuh"
 
@@ -30,11 +31,11 @@ constexpr int kMaxHalo = 64;
 constexpr int kMaxTable = 512;
 
 enum KernelId {
-  K_SWEEP_X, K_SWEEP_Y, K_SWEEP_Z, K_OBS, K_VMOM, K_VCOUNT, K_NORM, K_INIT, K_IO, K_TABLES,
+  K_SWEEP_X, K_SWEEP_Y, K_SWEEP_Z, K_OBS, K_NORM, K_INIT, K_IO, K_TABLES,
   K_XY, K_RESIDENT, K_COUNT
 };
 const char* kKernelNames[K_COUNT] = {"sweep_x_h1",  "sweep_y",        "sweep_z",
-                                     "observables", "vortex_moments", "vortex_count",
+                                     "observables",
                                      "norm",        "init_analytic",  "pack_unpack",
                                      "tables",      "xy_pass_h1",     "steps_2d"};
 
@@ -130,9 +131,11 @@ struct rotgp_ctx {
   double* partials = nullptr;
   size_t partial_doubles = 0;
   unsigned* counter = nullptr;
-  double* scalars = nullptr;  // [0] scale, [1] norm, [2..2+NOBS) obs, [+2] moments
-  int* iflags = nullptr;      // [0] flags, [1] vortex count
-  double* h_obs = nullptr;    // pinned: NOBS doubles + 2 ints
+  // [0] scale, [1] norm, [2 .. 2 + OS_COUNT) sums of the observables, then
+  // two ints: flags, vortex count (read back together)
+  double* scalars = nullptr;
+  int* iflags = nullptr;
+  double* h_obs = nullptr;    // pinned: OS_COUNT sums and the two ints
   size_t device_bytes = 0;
   long long steps = 0;
   std::string err;
@@ -146,8 +149,7 @@ struct rotgp_ctx {
 
   double* d_scale() { return scalars; }
   double* d_norm() { return scalars + 1; }
-  double* d_obs() { return scalars + 2; }
-  double* d_moments() { return scalars + 2 + NOBS; }
+  double* d_sums() { return scalars + 2; }
   int* d_flags() { return iflags; }
   int* d_count() { return iflags + 1; }
 };
@@ -962,12 +964,7 @@ bool schedule_tables(rotgp_ctx* c) {
   return true;
 }
 
-int check_flags(rotgp_ctx* c) {
-  int flags = 0;
-  cudaError_t e = cudaMemcpyAsync(&flags, c->d_flags(), sizeof(int), cudaMemcpyDeviceToHost,
-                                  c->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-  if (e != cudaSuccess) return cuda_fail(c, e, "synchronise");
+int flags_error(rotgp_ctx* c, int flags) {
   if (flags & 2) return fail(c, ROTGP_ECUDA, "a sweep kernel was launched with a shape it was not built for");
   if (flags & 4) return fail(c, ROTGP_ETIMEOUT, "a tile pass gave up waiting for its TMA load");
   if (flags & 8) {
@@ -978,6 +975,15 @@ int check_flags(rotgp_ctx* c) {
   }
   if (flags & 1) return fail(c, ROTGP_ENONFINITE, "non-finite or zero norm in a reduction");
   return ROTGP_OK;
+}
+
+int check_flags(rotgp_ctx* c) {
+  int flags = 0;
+  cudaError_t e = cudaMemcpyAsync(&flags, c->d_flags(), sizeof(int), cudaMemcpyDeviceToHost,
+                                  c->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+  if (e != cudaSuccess) return cuda_fail(c, e, "synchronise");
+  return flags_error(c, flags);
 }
 
 bool finite_phys(const rotgp_phys* p) {
@@ -1002,7 +1008,6 @@ void release(rotgp_ctx* c) {
   cudaFree(c->partials);
   cudaFree(c->counter);
   cudaFree(c->scalars);
-  cudaFree(c->iflags);
   if (c->h_obs) cudaFreeHost(c->h_obs);
   for (auto& r : c->recs) {
     cudaEventDestroy(r.a);
@@ -1083,6 +1088,80 @@ void ctx_get_view(const rotgp_ctx* c, ctx_view* v) {
   v->hx = c->grid.h[0];
   v->hy = c->grid.h[1];
   v->vol = c->vol;
+}
+
+// Enqueue the evaluation of the observables and the copy of its sums.
+int ctx_observe(rotgp_ctx* c) {
+  observe_args a{};
+  a.psi = c->psi[c->cur];
+  a.nx = c->nx;
+  a.ny = c->ny;
+  a.nz = c->nz;
+  a.dim = c->grid.dim;
+  a.kplane = c->grid.dim == 3 ? c->grid.n[2] / 2 : 0;
+  a.hx = c->grid.h[0];
+  a.hy = c->grid.h[1];
+  a.hz = c->grid.dim == 3 ? c->grid.h[2] : 0.0;
+  a.x0 = c->x0;
+  a.y0 = c->y0;
+  a.z0 = c->z0;
+  a.hgam2 = 0.5 * c->phys.gamma * c->phys.gamma;
+  a.hnu2 = 0.5 * c->phys.nu * c->phys.nu;
+  a.hlam2 = c->grid.dim == 3 ? 0.5 * c->phys.lambda * c->phys.lambda : 0.0;
+  a.omega = c->phys.omega;
+  a.scale = c->d_scale();
+  a.partials = c->partials;
+  a.counter = c->counter;
+  a.sums = c->d_sums();
+  a.count = c->d_count();
+  a.ellipse = reinterpret_cast<observe_ellipse*>(c->scalars + 2 + OS_COUNT + 1);
+  a.fx0 = (float)(c->x0 + 0.5 * a.hx);
+  a.fy0 = (float)(c->y0 + 0.5 * a.hy);
+  a.fhx = (float)a.hx;
+  a.fhy = (float)a.hy;
+  int blocks = 1;
+  observe_shape(c->nx, c->ny, c->nz, c->grid.dim, c->sm_count, &a.chunk, &blocks);
+  cudaError_t e;
+  {
+    Timed t(c, K_OBS);
+    e = launch_observe(c->fp64, a, blocks, c->stream);
+  }
+  if (e != cudaSuccess) return cuda_fail(c, e, "observables kernels");
+  e = cudaMemcpyAsync(c->h_obs, c->d_sums(), (OS_COUNT + 1) * sizeof(double),
+                      cudaMemcpyDeviceToHost, c->stream);
+  return e == cudaSuccess ? ROTGP_OK : cuda_fail(c, e, "copy observables");
+}
+
+// Wait for the sums of ctx_observe and form the observables.
+int ctx_observed(rotgp_ctx* c, rotgp_obs* out) {
+  const cudaError_t e = cudaStreamSynchronize(c->stream);
+  if (e != cudaSuccess) return cuda_fail(c, e, "synchronise");
+  int ints[2];
+  std::memcpy(ints, c->h_obs + OS_COUNT, sizeof ints);
+  const int rc = flags_error(c, ints[0]);
+  if (rc) return rc;
+  const double* q = c->h_obs;
+  const double s0 = q[OS_RE2] + q[OS_IM2], g = c->phys.g;
+  const bool rot = q[OS_RE2] < 1e-3 * s0;
+  const double lin = q[rot ? OS_LI : OS_LR], nl = g * q[rot ? OS_NI : OS_NR];
+  const double den = q[rot ? OS_IM2 : OS_RE2];
+  const double lin_c = q[OS_LR] + q[OS_LI], nl_c = g * (q[OS_NR] + q[OS_NI]);
+  out->norm = c->vol * s0;
+  out->mu = (lin + nl) / den;
+  out->energy = (lin + 0.5 * nl) / den;
+  out->mu_c = (lin_c + nl_c) / s0;
+  out->energy_c = (lin_c + 0.5 * nl_c) / s0;
+  out->rms_x = std::sqrt(q[OS_X2] / s0);
+  out->rms_y = std::sqrt(q[OS_Y2] / s0);
+  out->rms_z = c->grid.dim == 3 ? std::sqrt(q[OS_Z2] / s0) : 0.0;
+  out->rms_r = std::sqrt((q[OS_X2] + q[OS_Y2] + q[OS_Z2]) / s0);
+  out->max_density = q[OS_MAX];
+  out->mu4 = (q[OS_L4] + nl_c) / s0;
+  out->energy4 = (q[OS_L4] + 0.5 * nl_c) / s0;
+  out->vortices = ints[1];
+  out->step = c->steps;
+  out->flags = c->phys.omega >= std::min(c->phys.gamma, c->phys.nu) ? 1 : 0;
+  return ROTGP_OK;
 }
 
 // Message returned by rotgp_last_error(NULL) on this thread.
@@ -1189,7 +1268,8 @@ int rotgp_create(const rotgp_grid* grid, const rotgp_phys* phys, int precision, 
   c->axis[1].nlines = c->nx;
   c->axis[2].nlines = 1;
   // reduction scratch: the largest per-block partial count of any reduction
-  size_t pd = (size_t)reduce_blocks(c, c->sites) * NQ;
+  size_t pd = (size_t)std::max(reduce_blocks(c, c->sites), kObserveBlocksPerSm * c->sm_count) *
+              OS_COUNT;
   {
     // largest block count any launch shape of the last sweep can take:
     // one warp per block, one line per lane, one segment per chunk
@@ -1199,7 +1279,6 @@ int rotgp_create(const rotgp_grid* grid, const rotgp_phys* phys, int precision, 
     // the one-line-per-lane form groups lines by 32 consecutive x
     pd = std::max(pd, (size_t)strided1_blocks(last.lines, c->nx, (int)nch));
   }
-  pd = std::max(pd, (size_t)reduce_blocks(c, (long long)c->nx * c->ny) * 3);
   {
     // the exact partition solve of the last axis: one block per tile
     const int la = grid->dim - 1;
@@ -1245,9 +1324,10 @@ int rotgp_create(const rotgp_grid* grid, const rotgp_phys* phys, int precision, 
   }
   if (!rc) rc = dev_alloc(c, (void**)&c->partials, c->partial_doubles * sizeof(double));
   if (!rc) rc = dev_alloc(c, (void**)&c->counter, sizeof(unsigned));
-  if (!rc) rc = dev_alloc(c, (void**)&c->scalars, (2 + NOBS + 2) * sizeof(double));
-  if (!rc) rc = dev_alloc(c, (void**)&c->iflags, 2 * sizeof(int));
-  if (!rc && cudaMallocHost((void**)&c->h_obs, (NOBS + 2) * sizeof(double)) != cudaSuccess)
+  if (!rc) rc = dev_alloc(c, (void**)&c->scalars,
+                         (2 + OS_COUNT + 1) * sizeof(double) + sizeof(observe_ellipse));
+  if (!rc) c->iflags = reinterpret_cast<int*>(c->scalars + 2 + OS_COUNT);
+  if (!rc && cudaMallocHost((void**)&c->h_obs, (OS_COUNT + 1) * sizeof(double)) != cudaSuccess)
     rc = fail(c, ROTGP_ENOMEM, "pinned host allocation failed");
   if (!rc) {
     e = cudaMemsetAsync(c->psi[0], 0, state, c->stream);
@@ -1407,22 +1487,17 @@ int rotgp_set_psi(rotgp_ctx* c, const void* src, int src_on_device, int src_is_f
     if (e != cudaSuccess) return cuda_fail(c, e, "copy state to device");
     from = c->staging;
   }
-  {
-    Timed t(c, K_IO);
-    e = launch_pack(c->fp64, src_is_fp64 != 0, from, c->psi[c->cur], c->nx, c->ny, c->nz,
-                    c->grid.dim, c->d_scale(), c->stream);
-  }
-  if (e != cudaSuccess) return cuda_fail(c, e, "pack kernel");
   if ((e = cudaMemsetAsync(c->iflags, 0, sizeof(int), c->stream)) != cudaSuccess)
     return cuda_fail(c, e, "reset flags");
-  if (normalise) {
-    // the norm and the pending scale 1/sqrt(norm), as after an imaginary-time step
-    Timed t(c, K_NORM);
-    e = launch_norm(c->fp64, c->psi[c->cur], c->sites, c->vol, 1, c->partials, c->counter,
-                    c->d_scale(), c->d_norm(), c->d_flags(), reduce_blocks(c, c->sites), 256,
-                    c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "norm kernel");
+  {
+    // with normalise the norm and the pending scale 1/sqrt(norm), as after an
+    // imaginary-time step
+    Timed t(c, K_IO);
+    e = launch_load(c->fp64, src_is_fp64 != 0, from, c->psi[c->cur], c->nx, c->ny, c->nz,
+                    c->grid.dim, c->vol, normalise != 0, c->partials, c->counter, c->d_scale(),
+                    c->d_norm(), c->d_flags(), reduce_blocks(c, c->sites), c->stream);
   }
+  if (e != cudaSuccess) return cuda_fail(c, e, "load kernel");
   c->steps = 0;
   e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "set_psi");
@@ -1544,96 +1619,8 @@ int rotgp_step_schedule(rotgp_ctx* c, long long n, int imag, const double* omega
 
 int rotgp_observables(rotgp_ctx* c, rotgp_obs* out) {
   if (!c || !out) return c ? fail(c, ROTGP_EINVAL, "null output") : ROTGP_EINVAL;
-  obs_args a{};
-  a.psi = c->psi[c->cur];
-  a.nx = c->nx;
-  a.ny = c->ny;
-  a.nz = c->nz;
-  a.dim = c->grid.dim;
-  a.hx = c->grid.h[0];
-  a.hy = c->grid.h[1];
-  a.hz = c->grid.dim == 3 ? c->grid.h[2] : 0.0;
-  a.x0 = c->x0;
-  a.y0 = c->y0;
-  a.z0 = c->z0;
-  a.hgam2 = 0.5 * c->phys.gamma * c->phys.gamma;
-  a.hnu2 = 0.5 * c->phys.nu * c->phys.nu;
-  a.hlam2 = c->grid.dim == 3 ? 0.5 * c->phys.lambda * c->phys.lambda : 0.0;
-  a.g = c->phys.g;
-  a.omega = c->phys.omega;
-  a.scale = c->d_scale();
-  a.partials = c->partials;
-  a.counter = c->counter;
-  a.result = c->d_obs();
-  cudaError_t e;
-  {
-    // work items of 32 x 8 columns and a z range: split z until there are
-    // about reduce_blocks() items (at least 16 planes each), at most that
-    // many blocks (the partials buffer), items taken grid-stride
-    const long long tiles = (long long)((c->nx + 31) / 32) * ((c->ny + 7) / 8);
-    const long long want = reduce_blocks(c, c->sites);
-    const int nz = c->grid.dim == 3 ? c->nz : 1;
-    const long long zparts =
-        std::max(1LL, std::min<long long>((want + tiles - 1) / tiles, nz / 16));
-    a.zchunk = (int)((nz + zparts - 1) / zparts);
-    const long long items = tiles * ((nz + a.zchunk - 1) / a.zchunk);
-    const int blocks = (int)std::min(items, want);
-    Timed t(c, K_OBS);
-    e = launch_observables(c->fp64, a, blocks, 256, c->stream);
-  }
-  if (e != cudaSuccess) return cuda_fail(c, e, "observables kernel");
-  vort_args v{};
-  v.psi = c->psi[c->cur];
-  v.nx = c->nx;
-  v.ny = c->ny;
-  v.nz = c->nz;
-  v.dim = c->grid.dim;
-  v.kplane = c->grid.dim == 3 ? c->grid.n[2] / 2 : 0;
-  v.hx = c->grid.h[0];
-  v.hy = c->grid.h[1];
-  v.x0 = c->x0;
-  v.y0 = c->y0;
-  v.partials = c->partials;
-  v.counter = c->counter;
-  v.moments = c->d_moments();
-  v.count = c->d_count();
-  const int vb = reduce_blocks(c, (long long)c->nx * c->ny);
-  {
-    Timed t(c, K_VMOM);
-    e = launch_vortex_moments(c->fp64, v, vb, 256, c->stream);
-  }
-  if (e == cudaSuccess) {
-    Timed t(c, K_VCOUNT);
-    e = launch_vortex_count(c->fp64, v, vb, 256, c->stream);
-  }
-  if (e != cudaSuccess) return cuda_fail(c, e, "vortex kernels");
-  e = cudaMemcpyAsync(c->h_obs, c->d_obs(), NOBS * sizeof(double), cudaMemcpyDeviceToHost,
-                      c->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(c->h_obs + NOBS, c->d_count(), sizeof(int), cudaMemcpyDeviceToHost,
-                        c->stream);
-  if (e != cudaSuccess) return cuda_fail(c, e, "copy observables");
-  int rc = check_flags(c);
-  if (rc) return rc;
-  const double* r = c->h_obs;
-  out->norm = r[0];
-  out->mu = r[1];
-  out->energy = r[2];
-  out->mu_c = r[3];
-  out->energy_c = r[4];
-  out->rms_x = r[5];
-  out->rms_y = r[6];
-  out->rms_z = r[7];
-  out->rms_r = r[8];
-  out->max_density = r[9];
-  out->mu4 = r[10];
-  out->energy4 = r[11];
-  int cnt = 0;
-  std::memcpy(&cnt, c->h_obs + NOBS, sizeof(int));
-  out->vortices = cnt;
-  out->step = c->steps;
-  out->flags = c->phys.omega >= std::min(c->phys.gamma, c->phys.nu) ? 1 : 0;
-  return ROTGP_OK;
+  const int rc = rotgp::ctx_observe(c);
+  return rc ? rc : rotgp::ctx_observed(c, out);
 }
 
 int rotgp_sync(rotgp_ctx* c) {
