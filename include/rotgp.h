@@ -283,7 +283,10 @@ int rotgp_tune(rotgp_ctx* ctx, int axis, int lines_per_lane, int chunk, int ring
  * "steps_2d" of rotgp_profile_read, one record per launch); results equal
  * those of the sweeps up to float rounding and the same truncation bound.
  * A wait between its tiles is bounded (about 2 s of device time,
- * ROTGP_ETIMEOUT).
+ * ROTGP_ETIMEOUT).  Likewise imaginary-time steps in complex double with a
+ * halo of at most 64 points, shorter than the lines, run in kernels of their
+ * own (records "steps_2d" for whole blocks of 2D steps of lines up to 1024
+ * points, else the sweeps' names), equal to the sweeps up to rounding.
  * The y and z sweeps in stencil form, and the fused pass, stage their
  * tiles with TMA loads whose waits are bounded: a wait that runs out
  * (about 2 s) makes the next synchronising call return ROTGP_ETIMEOUT. */

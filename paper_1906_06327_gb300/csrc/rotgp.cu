@@ -17,6 +17,7 @@
 
 #include "../../include/rotgp.h"
 #include "common.cuh"
+#include "dsteps.cuh"
 #include "observe.cuh"
 #include "resident.cuh"
 #include "tma.cuh"
@@ -128,6 +129,12 @@ struct rotgp_ctx {
   float2* rsched[2] = {nullptr, nullptr};  // tables of kResSchedule steps, per axis
   unsigned long long* xbuf = nullptr;      // two exchange planes,
   res_sync* rsync = nullptr;               // ... the exchange words (and rtab) behind them
+  // imaginary time in complex double (dsteps.cu), while the plan is the
+  // default one: weights per axis, points per lane of the rows, own points of
+  // the columns' segments (0: not served); dsync for whole blocks of 2D steps
+  double2* dtab[3] = {nullptr, nullptr, nullptr};
+  int d_rows = 0, d_seg[3] = {0, 0, 0};
+  dsync* d_sync = nullptr;
   double* partials = nullptr;
   size_t partial_doubles = 0;
   unsigned* counter = nullptr;
@@ -670,25 +677,138 @@ int stencil_weights(rotgp_ctx* c) {
   return ROTGP_OK;
 }
 
+// The tables of one axis and mode: those of the sweeps, of the on-chip
+// stepper and of the complex-double steps.
+int axis_tables(rotgp_ctx* c, int a, int mode) {
+  AxisPlan& ap = c->axis[a];
+  ap.co[mode] = make_coef(a, mode, c->grid.h[a], c->phys.dt, c->phys.omega, nlines_u0(c, a),
+                          nlines_du(c, a));
+  Timed t(c, K_TABLES);
+  cudaError_t e = launch_tables(c->fp64, ap.table[mode], ap.tableT[mode], ap.nlines, c->lt,
+                                ap.co[mode], c->stream);
+  if (e == cudaSuccess && a < 2 && c->rtab[a][mode]) {
+    const res_omegas one{{1.0}};
+    e = launch_res_tables(c->rtab[a][mode], ap.nlines, c->lt, ap.co[mode], one, 1, c->stream);
+  }
+  if (e == cudaSuccess && mode == 1 && c->dtab[a])
+    e = launch_dtables(c->dtab[a], ap.nlines, c->halo, ap.co[mode], c->stream);
+  return e == cudaSuccess ? ROTGP_OK : cuda_fail(c, e, "table kernel");
+}
+
+// Work split of the complex-double steps for the present halo.
+void double_plan(rotgp_ctx* c) {
+  c->d_rows = 0;
+  if (!c->fp64 || !c->chunk_ok || !c->dtab[0] || c->halo > kDPow) return;
+  c->d_rows = drow_points(c->nx, c->halo);
+  for (int a = 1; a < c->grid.dim && c->d_rows; ++a) {
+    const AxisPlan& ap = c->axis[a];
+    c->d_seg[a] = dcol_segment(ap.len, ap.lines, c->halo, c->sm_count);
+    if (c->d_seg[a] < 1 ||
+        (size_t)dcol_blocks(c->nx, ap.lines, ap.len, c->d_seg[a]) > c->partial_doubles)
+      c->d_rows = 0;
+  }
+}
+
 int build_tables(rotgp_ctx* c) {
+  double_plan(c);
   for (int a = 0; a < c->grid.dim; ++a) {
-    AxisPlan& ap = c->axis[a];
-    ap.wtab_fresh = false;
+    c->axis[a].wtab_fresh = false;
     for (int mode = 0; mode < 2; ++mode) {
-      ap.co[mode] = make_coef(a, mode, c->grid.h[a], c->phys.dt, c->phys.omega,
-                              nlines_u0(c, a), nlines_du(c, a));
-      Timed t(c, K_TABLES);
-      cudaError_t e = launch_tables(c->fp64, ap.table[mode], ap.tableT[mode], ap.nlines, c->lt,
-                                    ap.co[mode], c->stream);
-      if (e == cudaSuccess && a < 2 && c->rtab[a][mode]) {
-        const res_omegas one{{1.0}};
-        e = launch_res_tables(c->rtab[a][mode], ap.nlines, c->lt, ap.co[mode], one, 1,
-                              c->stream);
-      }
-      if (e != cudaSuccess) return cuda_fail(c, e, "table kernel");
+      const int rc = axis_tables(c, a, mode);
+      if (rc) return rc;
     }
   }
   return stencil_weights(c);
+}
+
+// Do complex-double steps of this mode run in the kernels of dsteps.cu, and
+// 2D ones in whole blocks?
+bool double_steps(const rotgp_ctx* c, bool imag) {
+  return imag && c->fp64 && c->d_rows && !c->user_plan && c->chunk_ok;
+}
+bool double_blocks(const rotgp_ctx* c, bool imag) {
+  return double_steps(c, imag) && c->d_sync && dstep_fits(c->nx, c->ny, c->halo);
+}
+
+int double_block(rotgp_ctx* c, long long n) {
+  dstep_args a{};
+  a.psi[0] = static_cast<double2*>(c->psi[c->cur]);
+  a.psi[1] = static_cast<double2*>(c->psi[1 - c->cur]);
+  a.tabx = c->dtab[0];
+  a.taby = c->dtab[1];
+  a.nx = c->nx;
+  a.ny = c->ny;
+  a.halo = c->halo;
+  a.ex0 = (int)std::max(-300.0, std::min(300.0, std::floor(-std::log2(c->vol)) + 1.0));
+  a.dt = c->phys.dt;
+  a.g = c->phys.g;
+  a.hgam2 = 0.5 * c->phys.gamma * c->phys.gamma;
+  a.hnu2 = 0.5 * c->phys.nu * c->phys.nu;
+  a.x0 = c->x0;
+  a.hx = c->grid.h[0];
+  a.y0 = c->y0;
+  a.hy = c->grid.h[1];
+  a.vol = c->vol;
+  a.scale = c->d_scale();
+  a.norm = c->d_norm();
+  a.flags = c->d_flags();
+  a.sync = c->d_sync;
+  for (long long s = 0; s < n; s += a.nsteps) {
+    a.nsteps = (int)std::min<long long>(2048, n - s);
+    cudaError_t e;
+    {
+      Timed t(c, K_RESIDENT);
+      e = launch_dsteps(a, c->sm_count, c->stream);
+    }
+    if (e != cudaSuccess) return cuda_fail(c, e, "complex-double steps launch");
+    c->steps += a.nsteps;
+  }
+  return ROTGP_OK;
+}
+
+// One sweep of an imaginary-time step in complex double.
+int double_sweep(rotgp_ctx* c, int axis, bool last) {
+  const AxisPlan& ap = c->axis[axis];
+  dline_args a{};
+  a.in = static_cast<const double2*>(c->psi[c->cur]);
+  a.out = static_cast<double2*>(c->psi[1 - c->cur]);
+  a.tab = c->dtab[axis];
+  a.tlines = ap.nlines;
+  a.nx = c->nx;
+  a.ny = c->ny;
+  a.nz = c->nz;
+  a.axis = axis;
+  a.len = ap.len;
+  a.halo = c->halo;
+  a.lines = ap.lines;
+  a.seg = c->d_seg[axis];
+  a.dt = c->phys.dt;
+  a.g = c->phys.g;
+  a.hgam2 = 0.5 * c->phys.gamma * c->phys.gamma;
+  a.hnu2 = 0.5 * c->phys.nu * c->phys.nu;
+  a.hlam2 = c->grid.dim == 3 ? 0.5 * c->phys.lambda * c->phys.lambda : 0.0;
+  a.x0 = c->x0;
+  a.hx = c->grid.h[0];
+  a.y0 = c->y0;
+  a.hy = c->grid.h[1];
+  a.z0 = c->z0;
+  a.hz = c->grid.dim == 3 ? c->grid.h[2] : 0.0;
+  a.vol = c->vol;
+  a.imag = 1;
+  a.partials = c->partials;
+  a.counter = c->counter;
+  a.scale_out = c->d_scale();
+  a.norm_out = c->d_norm();
+  a.flags = c->d_flags();
+  a.scale = c->d_scale();
+  cudaError_t e;
+  {
+    Timed t(c, axis == 0 ? K_SWEEP_X : (axis == 1 ? K_SWEEP_Y : K_SWEEP_Z));
+    e = axis == 0 ? launch_drows(a, c->d_rows, c->stream) : launch_dcols(last, a, c->stream);
+  }
+  if (e != cudaSuccess) return cuda_fail(c, e, "complex-double sweep launch");
+  c->cur = 1 - c->cur;
+  return ROTGP_OK;
 }
 
 // Does a step of this mode run in the on-chip stepper?  2D complex float
@@ -921,6 +1041,8 @@ int run_steps(rotgp_ctx* c, long long n, bool imag) {
   if (!c) return ROTGP_EINVAL;
   if (n < 0) return fail(c, ROTGP_EINVAL, "negative step count");
   if (resident(c, imag)) return resident_steps(c, n, imag, nullptr);
+  if (double_blocks(c, imag)) return double_block(c, n);
+  const bool dbl = double_steps(c, imag);
   for (long long s = 0; s < n; ++s) {
     for (int a = 0; a < c->grid.dim; ++a) {
       int rc;
@@ -932,6 +1054,8 @@ int run_steps(rotgp_ctx* c, long long n, bool imag) {
       if (a == 0 && c->fuse_xy && imag) {
         rc = xy_pass(c, imag);
         ++a;  // the y sweep is part of the pass
+      } else if (dbl) {
+        rc = double_sweep(c, a, a == c->grid.dim - 1);
       } else {
         rc = sweep(c, a, imag, a == c->grid.dim - 1);
       }
@@ -968,10 +1092,13 @@ int flags_error(rotgp_ctx* c, int flags) {
   if (flags & 2) return fail(c, ROTGP_ECUDA, "a sweep kernel was launched with a shape it was not built for");
   if (flags & 4) return fail(c, ROTGP_ETIMEOUT, "a tile pass gave up waiting for its TMA load");
   if (flags & 8) {
-    // no tag of the abandoned steps may be taken for one of a later launch
-    cudaMemsetAsync(c->rsync, 0, sizeof(res_sync), c->stream);
-    cudaMemsetAsync(c->xbuf, 0, 4 * (size_t)c->sites * sizeof(unsigned long long), c->stream);
-    return fail(c, ROTGP_ETIMEOUT, "a tile of the on-chip stepper gave up waiting for the others");
+    // no tag or count of the abandoned steps may be taken for one of a later launch
+    if (c->rsync) {
+      cudaMemsetAsync(c->rsync, 0, sizeof(res_sync), c->stream);
+      cudaMemsetAsync(c->xbuf, 0, 4 * (size_t)c->sites * sizeof(unsigned long long), c->stream);
+    }
+    if (c->d_sync) cudaMemsetAsync(c->d_sync, 0, sizeof(dsync), c->stream);
+    return fail(c, ROTGP_ETIMEOUT, "a block of steps gave up: one of its CTAs did not arrive in time");
   }
   if (flags & 1) return fail(c, ROTGP_ENONFINITE, "non-finite or zero norm in a reduction");
   return ROTGP_OK;
@@ -1004,6 +1131,7 @@ void release(rotgp_ctx* c) {
     ap.wtab = nullptr;
   }
   for (float2*& p : c->rsched) cudaFree(p), p = nullptr;
+  cudaFree(c->dtab[0]);  // and the other axes' and the exchange words
   cudaFree(c->xbuf);  // and the exchange words and weights behind the planes
   cudaFree(c->partials);
   cudaFree(c->counter);
@@ -1062,7 +1190,9 @@ int encode_state_map(CUtensorMap* map, void* base, int nx, int ny, int nz, unsig
 int ctx_buffer(const rotgp_ctx* c) { return c->cur; }
 void ctx_set_buffer(rotgp_ctx* c, int cur) { c->cur = cur; }
 long long ctx_steps(const rotgp_ctx* c) { return c->steps; }
-bool ctx_resident(const rotgp_ctx* c, bool imag) { return resident(c, imag); }
+bool ctx_resident(const rotgp_ctx* c, bool imag) {
+  return resident(c, imag) || double_blocks(c, imag);
+}
 long long ctx_plan_version(const rotgp_ctx* c) { return c->plan_version; }
 void ctx_add_steps(rotgp_ctx* c, long long n) { c->steps += n; }
 void ctx_get_view(const rotgp_ctx* c, ctx_view* v) {
@@ -1286,6 +1416,12 @@ int rotgp_create(const rotgp_grid* grid, const rotgp_phys* phys, int precision, 
     if (last.hyb_ok)
       pd = std::max(pd, (size_t)(hybrid_groups(la, last.lines, c->nx) * 8));
   }
+  if (c->fp64) {
+    // ... of the last axis' segments in complex double
+    const AxisPlan& last = c->axis[grid->dim - 1];
+    const int seg = c->halo <= kDPow ? dcol_segment(last.len, last.lines, c->halo, c->sm_count) : 0;
+    if (seg) pd = std::max(pd, (size_t)dcol_blocks(c->nx, last.lines, last.len, seg));
+  }
   c->partial_doubles = pd;
   c->staging_bytes = (size_t)(grid->n[0] + 1) * (grid->n[1] + 1) *
                      (grid->dim == 3 ? grid->n[2] + 1 : 1) * 16;
@@ -1358,6 +1494,22 @@ int rotgp_create(const rotgp_grid* grid, const rotgp_phys* phys, int precision, 
         e = cudaMemsetAsync(c->xbuf, 0, planes + sync, c->stream);
         if (e != cudaSuccess) rc = cuda_fail(c, e, "initialise buffers");
       }
+    }
+  }
+  if (!rc && c->fp64 && c->chunk_ok && c->halo <= kDPow) {
+    size_t lines = 0;
+    for (int a = 0; a < grid->dim; ++a) lines += c->axis[a].nlines;
+    double2* t = nullptr;
+    const size_t bytes = lines * kDPlanes * sizeof(double2);
+    rc = dev_alloc(c, (void**)&t, bytes + sizeof(dsync));
+    if (!rc) {
+      for (int a = 0; a < grid->dim; ++a) {
+        c->dtab[a] = t;
+        t += (size_t)kDPlanes * c->axis[a].nlines;
+      }
+      if (grid->dim == 2) c->d_sync = reinterpret_cast<dsync*>(t);
+      e = cudaMemsetAsync(t, 0, sizeof(dsync), c->stream);
+      if (e != cudaSuccess) rc = cuda_fail(c, e, "initialise buffers");
     }
   }
   if (!rc) build_maps(c);
@@ -1599,14 +1751,9 @@ int rotgp_step_schedule(rotgp_ctx* c, long long n, int imag, const double* omega
       // the x and y tables of this mode (z lines carry no rotation term)
       c->phys.omega = omega[k];
       for (int a = 0; a < 2; ++a) {
-        AxisPlan& ap = c->axis[a];
-        ap.co[mode] = make_coef(a, mode, c->grid.h[a], c->phys.dt, c->phys.omega,
-                                nlines_u0(c, a), nlines_du(c, a));
-        Timed t(c, K_TABLES);
-        cudaError_t e = launch_tables(c->fp64, ap.table[mode], ap.tableT[mode], ap.nlines, c->lt,
-                                      ap.co[mode], c->stream);
-        if (e != cudaSuccess) return cuda_fail(c, e, "table kernel");
-        ap.wtab_fresh = false;
+        const int rc = axis_tables(c, a, mode);
+        if (rc) return rc;
+        c->axis[a].wtab_fresh = false;
       }
     }
     int rc = imag ? stencil_weights(c) : ROTGP_OK;
@@ -1900,11 +2047,12 @@ int rotgp_autotune(rotgp_ctx* c, int steps, int* choice) {
     }
     ap.lsegs = best_s;
   }
-  // and the on-chip 2D stepper, which takes no form or shape
+  // and the on-chip 2D stepper or the complex-double kernels, which take no
+  // form or shape
   if (e == cudaSuccess && !rc) {
     c->user_plan = false;
     float ms = 0;
-    if (resident(c, true) && time_current(&ms) && ms < best_ms)
+    if ((resident(c, true) || double_steps(c, true)) && time_current(&ms) && ms < best_ms)
       best = 0;
     else
       c->user_plan = true;
