@@ -144,6 +144,9 @@ struct rotgp_ctx {
   int* iflags = nullptr;
   double* h_obs = nullptr;    // pinned: OS_COUNT sums and the two ints
   size_t device_bytes = 0;
+  std::vector<void*> blocks;   // allocations, and what is left of the last shared one
+  char* block_next = nullptr;
+  size_t block_left = 0;
   long long steps = 0;
   std::string err;
   // profiling
@@ -1121,21 +1124,9 @@ bool finite_phys(const rotgp_phys* p) {
 }
 
 void release(rotgp_ctx* c) {
-  for (void*& p : c->psi) cudaFree(p), p = nullptr;
-  cudaFree(c->staging);
-  cudaFree(c->dR);
-  for (auto& ap : c->axis) {
-    for (void*& t : ap.table) cudaFree(t), t = nullptr;
-    for (void*& t : ap.tableT) cudaFree(t), t = nullptr;
-    cudaFree(ap.wtab);
-    ap.wtab = nullptr;
-  }
+  for (void* p : c->blocks) cudaFree(p);
+  c->blocks.clear();
   for (float2*& p : c->rsched) cudaFree(p), p = nullptr;
-  cudaFree(c->dtab[0]);  // and the other axes' and the exchange words
-  cudaFree(c->xbuf);  // and the exchange words and weights behind the planes
-  cudaFree(c->partials);
-  cudaFree(c->counter);
-  cudaFree(c->scalars);
   if (c->h_obs) cudaFreeHost(c->h_obs);
   for (auto& r : c->recs) {
     cudaEventDestroy(r.a);
@@ -1144,13 +1135,30 @@ void release(rotgp_ctx* c) {
   for (auto e : c->pool) cudaEventDestroy(e);
 }
 
+// Device memory of the context, given back with it.  Small requests share
+// blocks of 1 MB: creating a context is mostly the time of its allocations.
 int dev_alloc(rotgp_ctx* c, void** p, size_t bytes) {
-  cudaError_t e = cudaMalloc(p, bytes);
-  if (e != cudaSuccess) {
-    *p = nullptr;
-    return fail(c, ROTGP_ENOMEM, "cudaMalloc(%zu): %s", bytes, cudaGetErrorString(e));
+  constexpr size_t kBlock = 1 << 20;
+  const size_t want = (bytes + 255) & ~(size_t)255;
+  if (want <= c->block_left) {
+    *p = c->block_next;
+  } else {
+    const size_t size = want <= kBlock / 2 ? kBlock : want;
+    void* q = nullptr;
+    const cudaError_t e = cudaMalloc(&q, size);
+    if (e != cudaSuccess) {
+      *p = nullptr;
+      return fail(c, ROTGP_ENOMEM, "cudaMalloc(%zu): %s", size, cudaGetErrorString(e));
+    }
+    c->blocks.push_back(q);
+    c->device_bytes += size;
+    *p = q;
+    if (size == want) return ROTGP_OK;
+    c->block_next = static_cast<char*>(q);
+    c->block_left = size;
   }
-  c->device_bytes += bytes;
+  c->block_next += want;
+  c->block_left -= want;
   return ROTGP_OK;
 }
 
