@@ -286,7 +286,10 @@ int rotgp_tune(rotgp_ctx* ctx, int axis, int lines_per_lane, int chunk, int ring
  * ROTGP_ETIMEOUT).  Likewise imaginary-time steps in complex double with a
  * halo of at most 64 points, shorter than the lines, run in kernels of their
  * own (records "steps_2d" for whole blocks of 2D steps of lines up to 1024
- * points, else the sweeps' names), equal to the sweeps up to rounding.
+ * points, else the sweeps' names), equal to the sweeps up to rounding; and
+ * complex-float sweeps with a halo of 17 to 64 points, or with odd N_x, take
+ * truncated tiles of lines instead of the forms named above, with results
+ * equal up to rounding and the truncation bound.
  * The y and z sweeps in stencil form, and the fused pass, stage their
  * tiles with TMA loads whose waits are bounded: a wait that runs out
  * (about 2 s) makes the next synchronising call return ROTGP_ETIMEOUT. */

@@ -133,11 +133,15 @@ int run_set_inner(rotgp_batch* b, const std::vector<int>& set, long long n, bool
   if (mode == ROTGP_BATCH_PERSISTENT) {
     const int count = (int)b->ctx.size();
     std::vector<rotgp::ctx_view> v(count);
-    for (int i = 0; i < count; ++i) rotgp::ctx_get_view(b->ctx[i], &v[i]);
+    std::vector<int> reach(count);
+    for (int i = 0; i < count; ++i) {
+      rotgp::ctx_get_view(b->ctx[i], &v[i]);
+      reach[i] = rotgp::ctx_carry_reach(b->ctx[i]);
+    }
     const char* why = "";
     if (!rotgp::batch_kernel_fits(v.data(), count, 200 * 1024, &why))
       return bfail(b, ROTGP_EUNSUPPORTED, "persistent batch step: %s", why);
-    e = rotgp::batch_kernel_run(&b->dev, v.data(), count, set.data(), (int)set.size(), n, imag,
+    e = rotgp::batch_kernel_run(&b->dev, v.data(), reach.data(), count, set.data(), (int)set.size(), n, imag,
                                 b->stream);
     if (e != cudaSuccess)
       return bfail(b, ROTGP_ECUDA, "persistent batch launch: %s", cudaGetErrorString(e));

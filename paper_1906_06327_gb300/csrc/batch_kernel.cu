@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "hybrid.cuh"
+#include "resident.cuh"
 
 namespace rotgp {
 
@@ -38,6 +39,7 @@ struct binst {
   double* norm;
   int* flags;
   int nx, ny, lt, cur;
+  int reach;              // points in which a carry is above rounding
   int pcx, lsx, pcy, lsy;  // whole-line tile shapes of the x and y sweeps
   int ytile0, ytiles;      // this instance's slots of the norm partials
   int vec;
@@ -136,7 +138,7 @@ __device__ double partials_sum(const double* p, int n) {
 }
 
 template <class T, bool IMAG>
-__global__ void __launch_bounds__(kHThreads, sizeof(T) == 4 ? 2 : 1) k_batch_steps(const batch_args b) {
+__global__ void __launch_bounds__(kHThreads, sizeof(T) == 4 ? 3 : 1) k_batch_steps(const batch_args b) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   for (long long step = 0; step < b.nsteps; ++step) {
     // ---- phase X: H1 (with the pending scale) and the x sweep
@@ -155,6 +157,7 @@ __global__ void __launch_bounds__(kHThreads, sizeof(T) == 4 ? 2 : 1) k_batch_ste
       a.out = I.psi[1 - I.cur];
       a.coef = I.tab[0][IMAG ? 1 : 0];
       a.len = I.nx;
+      a.halo = I.reach;
       a.lt = I.lt;
       a.nlines = I.ny;
       a.nx = I.nx;
@@ -190,6 +193,7 @@ __global__ void __launch_bounds__(kHThreads, sizeof(T) == 4 ? 2 : 1) k_batch_ste
       a.out = I.psi[I.cur];
       a.coef = I.tab[1][IMAG ? 1 : 0];
       a.len = I.ny;
+      a.halo = I.reach;
       a.lt = I.lt;
       a.nlines = I.nx;
       a.nx = I.nx;
@@ -304,7 +308,8 @@ bool batch_kernel_fits(const ctx_view* v, int count, size_t smem_limit, const ch
   return true;
 }
 
-cudaError_t batch_kernel_run(batch_dev** dp, const ctx_view* v, int count, const int* active,
+cudaError_t batch_kernel_run(batch_dev** dp, const ctx_view* v, const int* reach, int count,
+                             const int* active,
                              int nact, long long nsteps, bool imag, cudaStream_t s) {
   if (!*dp) *dp = new batch_dev();
   batch_dev& d = **dp;
@@ -324,6 +329,7 @@ cudaError_t batch_kernel_run(batch_dev** dp, const ctx_view* v, int count, const
     I.nx = v[i].nx;
     I.ny = v[i].ny;
     I.lt = v[i].lt;
+    I.reach = reach[i];
     I.cur = v[i].cur;
     smem = std::max(smem, hybrid_tile(I.nx, 0, fp64, 1, &I.pcx, &I.lsx));
     smem = std::max(smem, hybrid_tile(I.ny, 1, fp64, 1, &I.pcy, &I.lsy));

@@ -15,8 +15,11 @@
 // X = x at the segment start).  The true carry into every segment follows by
 // composing the summaries of the segments before it (forward) or after it
 // (backward), which is the reduced system of the partition method, solved
-// here by direct composition; the segments then rerun their recurrences from
-// the true carries.  Nothing is truncated: the result is the Thomas solution
+// here by direct composition; the segments then add what the true carry adds
+// to their local solution, the products of the multipliers times it, over the
+// points in which that is above a thousandth of the rounding (rerunning both
+// recurrences from the true carries, as before, doubled the instructions: a
+// 4096^2 step 411 / 307 us, a step of the 64-instance batch 196 / 173 us).  Nothing is truncated: the result is the Thomas solution
 // of the whole line up to rounding, whatever the decay of the carries.
 //
 // Layout.  A CTA of 256 threads holds a tile of 16 lines x pc positions (+2
@@ -34,7 +37,7 @@
 // measured slower on GB300: 3.0e10 against 3.3e10 site-updates/s on the 4096^2
 // state, 241 against 196 us per persistent batch step).  Each point is read from and written to global
 // memory once per sweep; H1 (with the pending renormalisation) is applied to
-// the tile as it lands in the x sweep; the last sweep of a step reduces the
+// each point as the x sweep's forward pass reaches it; the last sweep of a step reduces the
 // norm.  The same kernel serves both propagation modes (the table of the mode
 // is passed) and both precisions.
 #include "hybrid.cuh"
@@ -44,7 +47,7 @@
 namespace rotgp {
 
 template <class T, int AX, bool H1, bool IMAG, bool REDUCE>
-__global__ void __launch_bounds__(kHThreads, sizeof(T) == 4 ? 2 : 1) k_line_hybrid(const hybrid_args ha) {
+__global__ void __launch_bounds__(kHThreads, sizeof(T) == 4 ? 3 : 1) k_line_hybrid(const hybrid_args ha) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   hybrid_job J;
   J.cs = ha.cs;

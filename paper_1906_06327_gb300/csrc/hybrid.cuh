@@ -113,7 +113,7 @@ __device__ __forceinline__ double hybrid_tile(const stream_args& a, const hybrid
   __shared__ T hv[kHL];
 
   cg::cluster_group cluster = cg::this_cluster();
-  const int cs = J.cs, pc = J.pc, lsub = J.lsub, rank = J.rank;
+  const int cs = J.cs, pc = J.pc, lsub = J.lsub, rank = J.rank, reach = a.halo;
   // a tile of whole lines (cs = 1) runs without a cluster: no cluster
   // barrier and no remote shared memory then
   auto csync = [&]() {
@@ -151,16 +151,16 @@ __device__ __forceinline__ double hybrid_tile(const stream_args& a, const hybrid
   };
 
   // ---- load the tile (zeros outside the grid and past the line end), ep
-  // complex numbers per copy
+  // complex numbers per copy; x lines by warps, a row each
   auto load = [&](auto ep_tag) {
     constexpr int ep = decltype(ep_tag)::value;
     if (AX == 0) {
-      for (int l = 0; l < kHL; ++l) {
+      for (int l = tid >> 5; l < kHL; l += kHThreads / 32) {
         const bool ok = line_ok(l);
         const E* src = in + (grp * kHL + l) * (long long)N;
         E* dst = tile + l * W;
-        for (int c = tid; c < W / ep; c += kHThreads) {
-          const int e = c * ep, p = p0 - 2 + e;
+        for (int e = (tid & 31) * ep; e < W; e += 32 * ep) {
+          const int p = p0 - 2 + e;
           if (ok && p >= 0 && p + ep <= N) {
             cp_async<ep * sizeof(E)>(dst + e, src + p);
           } else {
@@ -199,29 +199,12 @@ __device__ __forceinline__ double hybrid_tile(const stream_args& a, const hybrid
   cp_async_wait<0>();
   __syncthreads();
 
-  // ---- H1 with the pending renormalisation (x sweep): psi <- s psi, then
-  // exp(-Delta (V + g|psi|^2)) or exp(-i Delta (V + g|psi|^2)) (Eq. eq1).
-  // Imaginary time advances the tile in place.  Real time leaves it as
-  // loaded: each forward pass forms every point as value + increment (hpt)
-  // when it reaches it.
+  // H1 with the pending renormalisation (x sweep), applied to each point as
+  // the forward pass reaches it: psi <- s psi, then exp(-Delta (V + g|psi|^2))
+  // or, as value and increment (hpt), exp(-i Delta (V + g|psi|^2)) (Eq. eq1).
   constexpr bool RT = H1 && !IMAG;
   const T h_s = (T)J.scale, h_gg = (T)a.g, h_dt = (T)a.dt;
   const T h_hg2 = (T)a.hgam2, h_xs = (T)a.x0, h_hx = (T)a.hx;
-  if (H1 && IMAG) {
-    const T s = (T)J.scale, hg2 = (T)a.hgam2, gg = (T)a.g, dt = (T)a.dt;
-    const T xs = (T)a.x0, hx = (T)a.hx;
-    for (int l = 0; l < kHL; ++l) {
-      const T vyz = hv[l];
-      E* row = tile + l * W;
-      for (int e = tid; e < W; e += kHThreads) {
-        const T x = fma((T)(p0 - 2 + e), hx, xs);
-        E v = rscale(s, row[e]);
-        const T en = fma(gg, sq(v), fma(hg2 * x, x, vyz));
-        row[e] = rscale(exp_t(-dt * en), v);
-      }
-    }
-    __syncthreads();
-  }
 
   // ---- this thread's line and sub-segment
   const int l = AX == 0 ? tid / kHS : tid % kHL;
@@ -238,60 +221,64 @@ __device__ __forceinline__ double hybrid_tile(const stream_args& a, const hybrid
   // the scan threads: a half-warp over the sub-segments of one line
   const int l2 = tid / kHS, k2 = tid % kHS;
 
-  // real time: the loaded value u of tile position e of this thread's line,
-  // scaled and advanced
-  auto rt_at = [&](E u, int e) -> hpt<T> {
+  // the loaded value u of tile position e of this thread's line, scaled and
+  // advanced
+  auto energy = [&](E v, int e) -> T {
     const T x = fma((T)(p0 - 2 + e), h_hx, h_xs);
+    return fma(h_gg, sq(v), fma(h_hg2 * x, x, hv[AX == 0 ? l : 0]));
+  };
+  auto adv = [&](E u, int e) -> E {
+    if (!H1) return u;
     const E v = rscale(h_s, u);
-    const T en = fma(h_gg, sq(v), fma(h_hg2 * x, x, hv[AX == 0 ? l : 0]));
+    return rscale(exp_t(-h_dt * energy(v, e)), v);
+  };
+  auto rt_at = [&](E u, int e) -> hpt<T> {
+    const E v = rscale(h_s, u);
     T c1, s1;
-    rot_t(h_dt * en, &c1, &s1);
+    rot_t(h_dt * energy(v, e), &c1, &s1);
     return rot_inc(v, c1, s1);
   };
-  auto rt = [&](int e) -> hpt<T> { return rt_at(el(l, e), e); };
 
-  // ---- F1: local forward from a zero carry; summary (prod al, d at the end)
+  // ---- forward from a zero carry, d over psi in the tile; summary (prod al,
+  // d at the end).  The neighbours outside the sub-segment are read first:
+  // the adjacent threads overwrite them.
   const E left = el(l, eb - 1), right = el(l, eb + nv);
-  if constexpr (RT) {
+  __syncthreads();
+  {
     E d = zero<T>(), G = mk<T>(1, 0);
-    E pm = hw(rt_at(left, eb - 1));
-    hpt<T> pc = rt(eb);
     int i = 0;
-    for (; i < it; ++i) {
-      const hpt<T> pn = i + 1 < nv ? rt(eb + i + 1) : rt_at(right, eb + nv);
-      d = fwd_inc(crow[pb + i], pm, pc, hw(pn), d);
-      G = cmul(crow[pb + i].al, G);
-      pm = hw(pc);
-      pc = pn;
-    }
+    if constexpr (RT) {
+      E pm = hw(rt_at(left, eb - 1));
+      hpt<T> pc = rt_at(el(l, eb), eb);
+      auto step = [&](const coef5<T>& c) {
+        const hpt<T> pn = rt_at(i + 1 < nv ? el(l, eb + i + 1) : right, eb + i + 1);
+        d = fwd_inc(c, pm, pc, hw(pn), d);
+        el(l, eb + i) = d;
+        pm = hw(pc);
+        pc = pn;
+      };
+      for (; i < it; ++i) {
+        step(crow[pb + i]);
+        G = cmul(crow[pb + i].al, G);
+      }
 #pragma unroll 2
-    for (; i < nv; ++i) {
-      const hpt<T> pn = i + 1 < nv ? rt(eb + i + 1) : rt_at(right, eb + nv);
-      d = fwd_inc(cinf, pm, pc, hw(pn), d);
-      pm = hw(pc);
-      pc = pn;
-    }
-    if (nv > it) G = cmul(G, cpow_n(cinf.al, nv - it));
-    sG[l][k] = G;
-    sD[l][k] = d;
-  } else {
-    E d = zero<T>(), G = mk<T>(1, 0);
-    E pm = left, pcur = el(l, eb);
-    int i = 0;
-    for (; i < it; ++i) {
-      const coef5<T> c = crow[pb + i];
-      const E pn = el(l, eb + i + 1);
-      d = fwd(c, pm, pcur, pn, d);
-      G = cmul(c.al, G);
-      pm = pcur;
-      pcur = pn;
-    }
+      for (; i < nv; ++i) step(cinf);
+    } else {
+      E pm = adv(left, eb - 1), pc = adv(el(l, eb), eb);
+      auto step = [&](const coef5<T>& c) {
+        const E pn = adv(i + 1 < nv ? el(l, eb + i + 1) : right, eb + i + 1);
+        d = fwd(c, pm, pc, pn, d);
+        el(l, eb + i) = d;
+        pm = pc;
+        pc = pn;
+      };
+      for (; i < it; ++i) {
+        const coef5<T> c = crow[pb + i];
+        step(c);
+        G = cmul(c.al, G);
+      }
 #pragma unroll 4
-    for (; i < nv; ++i) {
-      const E pn = el(l, eb + i + 1);
-      d = fwd(cinf, pm, pcur, pn, d);
-      pm = pcur;
-      pcur = pn;
+      for (; i < nv; ++i) step(cinf);
     }
     if (nv > it) G = cmul(G, cpow_n(cinf.al, nv - it));
     sG[l][k] = G;
@@ -334,63 +321,37 @@ __device__ __forceinline__ double hybrid_tile(const stream_args& a, const hybrid
   }
   __syncthreads();
 
-  // ---- F2: forward from the true carry; d overwrites psi in the tile
-  if constexpr (RT) {
-    // the neighbours outside the sub-segment come from the values read
-    // before the barrier: the adjacent sub-segments overwrite them in this
-    // pass (inside it, the read of eb + i + 1 precedes the store at eb + i + 1)
-    E d = sD[l][k];
-    E pm = hw(rt_at(left, eb - 1));
-    hpt<T> pc = rt(eb);
-    const hpt<T> rend = rt_at(right, eb + nv);
+  // ---- the true carry: d_p += (product of al) carry over the `reach` points
+  // in which it is above rounding
+  {
+    E c = sD[l][k];
+    const int n = min(nv, reach);
     int i = 0;
-    for (; i < it; ++i) {
-      const hpt<T> pn = i + 1 < nv ? rt(eb + i + 1) : rend;
-      d = fwd_inc(crow[pb + i], pm, pc, hw(pn), d);
-      el(l, eb + i) = d;
-      pm = hw(pc);
-      pc = pn;
-    }
-#pragma unroll 2
-    for (; i < nv; ++i) {
-      const hpt<T> pn = i + 1 < nv ? rt(eb + i + 1) : rend;
-      d = fwd_inc(cinf, pm, pc, hw(pn), d);
-      el(l, eb + i) = d;
-      pm = hw(pc);
-      pc = pn;
-    }
-  } else {
-    E d = sD[l][k];
-    E pm = left, pcur = el(l, eb);
-    int i = 0;
-    for (; i < it; ++i) {
-      const coef5<T> c = crow[pb + i];
-      const E pn = i + 1 < nv ? el(l, eb + i + 1) : right;
-      d = fwd(c, pm, pcur, pn, d);
-      el(l, eb + i) = d;
-      pm = pcur;
-      pcur = pn;
+    for (; i < min(n, it); ++i) {
+      c = cmul(crow[pb + i].al, c);
+      el(l, eb + i) = el(l, eb + i) + c;
     }
 #pragma unroll 4
-    for (; i < nv; ++i) {
-      const E pn = i + 1 < nv ? el(l, eb + i + 1) : right;
-      d = fwd(cinf, pm, pcur, pn, d);
-      el(l, eb + i) = d;
-      pm = pcur;
-      pcur = pn;
+    for (; i < n; ++i) {
+      c = cmul(cinf.al, c);
+      el(l, eb + i) = el(l, eb + i) + c;
     }
   }
-  // ---- B1: local backward from a zero carry; summary (prod be, x at the start)
+  // ---- backward from a zero carry, x over d; summary (prod be, x at the start)
   {
     E x = zero<T>(), B = mk<T>(1, 0);
     int i = nv - 1;
 #pragma unroll 4
-    for (; i >= it; --i) x = bwd(cinf.be, x, el(l, eb + i));
+    for (; i >= it; --i) {
+      x = bwd(cinf.be, x, el(l, eb + i));
+      el(l, eb + i) = x;
+    }
     if (nv > it) B = cpow_n(cinf.be, nv - it);
     for (; i >= 0; --i) {
-      const coef5<T> c = crow[pb + i];
-      x = bwd(c.be, x, el(l, eb + i));
-      B = cmul(c.be, B);
+      const E be = crow[pb + i].be;
+      x = bwd(be, x, el(l, eb + i));
+      el(l, eb + i) = x;
+      B = cmul(be, B);
     }
     __syncthreads();  // every thread has read its forward carry
     sG[l][k] = B;
@@ -433,44 +394,51 @@ __device__ __forceinline__ double hybrid_tile(const stream_args& a, const hybrid
   // every CTA's remote reads are done before any CTA moves on (and exits)
   csync();
 
-  // ---- B2: backward from the true carry; x overwrites d in the tile
-  acc_t<T> acc;
+  // ---- the true carry: x_p += (product of be) carry, from the end
   {
-    E x = sD[l][k];
+    E c = sD[l][k];
+    const int n0 = max(0, nv - reach);
     int i = nv - 1;
 #pragma unroll 4
-    for (; i >= it; --i) {
-      x = bwd(cinf.be, x, el(l, eb + i));
-      el(l, eb + i) = x;
-      if (REDUCE) acc.add(sq(x));
+    for (; i >= max(n0, it); --i) {
+      c = cmul(cinf.be, c);
+      el(l, eb + i) = el(l, eb + i) + c;
     }
-    for (; i >= 0; --i) {
-      const coef5<T> c = crow[pb + i];
-      x = bwd(c.be, x, el(l, eb + i));
-      el(l, eb + i) = x;
-      if (REDUCE) acc.add(sq(x));
+    for (; i >= n0; --i) {
+      c = cmul(crow[pb + i].be, c);
+      el(l, eb + i) = el(l, eb + i) + c;
     }
   }
   __syncthreads();
+  acc_t<T> acc;
 
   // ---- store the tile's own positions
   auto store = [&](auto ep_tag) {
     constexpr int ep = decltype(ep_tag)::value;
+    auto one = [&](E* dst, const E* src, bool both, bool first, bool second) {
+      if (ep == 2 && both) {
+        const float4 v = *reinterpret_cast<const float4*>(src);
+        *reinterpret_cast<float4*>(dst) = v;
+        if (REDUCE) acc.add(fmaf(v.x, v.x, v.y * v.y)), acc.add(fmaf(v.z, v.z, v.w * v.w));
+        return;
+      }
+      if (first) {
+        dst[0] = src[0];
+        if (REDUCE) acc.add(sq(src[0]));
+      }
+      if (ep == 2 && second) {
+        dst[1] = src[1];
+        if (REDUCE) acc.add(sq(src[1]));
+      }
+    };
     if (AX == 0) {
-      for (int ln = 0; ln < kHL; ++ln) {
+      for (int ln = tid >> 5; ln < kHL; ln += kHThreads / 32) {
         if (!line_ok(ln)) continue;
         E* dst = out + (grp * kHL + ln) * (long long)N;
         const E* row = tile + ln * W;
-        for (int c = tid; c < pc / ep; c += kHThreads) {
-          const int e = 2 + c * ep, p = p0 - 2 + e;
-          if (p >= N) continue;
-          if (ep == 2 && p + 1 < N) {
-            *reinterpret_cast<float4*>(dst + p) = *reinterpret_cast<const float4*>(row + e);
-          } else {
-#pragma unroll
-            for (int q = 0; q < ep; ++q)
-              if (p + q < N) dst[p + q] = row[e + q];
-          }
+        for (int c = (tid & 31) * ep; c < pc; c += 32 * ep) {
+          const int p = p0 + c;
+          one(dst + p, row + c + 2, p + 1 < N, p < N, p + 1 < N);
         }
       }
     } else {
@@ -478,14 +446,7 @@ __device__ __forceinline__ double hybrid_tile(const stream_args& a, const hybrid
       for (int u = tid; u < pc * per; u += kHThreads) {
         const int e = 2 + u / per, ln = (u % per) * ep, p = p0 - 2 + e;
         if (p >= N) continue;
-        if (ep == 2 && line_ok(ln + 1)) {
-          *reinterpret_cast<float4*>(out + gidx(ln, p)) =
-              *reinterpret_cast<const float4*>(&el(ln, e));
-        } else {
-#pragma unroll
-          for (int q = 0; q < ep; ++q)
-            if (line_ok(ln + q)) out[gidx(ln + q, p)] = el(ln + q, e);
-        }
+        one(out + gidx(ln, p), &el(ln, e), line_ok(ln + 1), line_ok(ln), line_ok(ln + 1));
       }
     }
   };

@@ -59,7 +59,7 @@
 #include <cmath>
 
 #include "resident.cuh"
-#include "sweep_common.cuh"
+#include "tail_solve.cuh"
 
 namespace rotgp {
 
@@ -152,23 +152,6 @@ __device__ __forceinline__ long long poll_total(const unsigned long long* word, 
   }
 }
 
-// ---------------------------------------------------------------- line solve
-// The weights of one line.
-struct line_w {
-  float2 al, be, g2, gc;
-};
-// k (v + r): the next value of a tail
-__device__ __forceinline__ float2 tail(float2 k, float2 v, float2 r) {
-  const float x = v.x + r.x, y = v.y + r.y;
-  return make_float2(fmaf(k.x, x, -(k.y * y)), fmaf(k.x, y, k.y * x));
-}
-// gc psi + g2 (f + b)
-__device__ __forceinline__ float2 change(const line_w& k, float2 psi, float2 f, float2 b) {
-  const float x = f.x + b.x, y = f.y + b.y;
-  return make_float2(
-      fmaf(k.g2.x, x, fmaf(-k.g2.y, y, fmaf(k.gc.x, psi.x, -(k.gc.y * psi.y)))),
-      fmaf(k.g2.x, y, fmaf(k.g2.y, x, fmaf(k.gc.x, psi.y, k.gc.y * psi.x))));
-}
 // The change of the L own points of a segment from its points w (H before,
 // L own, H after), p0 the position of w[0] on a line of N points; at(e): w[e]
 // for a run-time e.
@@ -207,37 +190,6 @@ __device__ __forceinline__ void solve_segment(const line_w& k, float2 (&w)[2 * H
     b = tail(k.be, w[H + i], b);
   }
 }
-// e^u - 1 to float accuracy relative to u: the Taylor series below 1/4, where
-// the steps of practice lie, and exp beyond.
-__device__ __forceinline__ float exp_m1(float u) {
-  float p = fmaf(u, 1.f / 5040.f, 1.f / 720.f);
-  p = fmaf(u, p, 1.f / 120.f);
-  p = fmaf(u, p, 1.f / 24.f);
-  p = fmaf(u, p, 1.f / 6.f);
-  p = fmaf(u, p, 0.5f);
-  p = fmaf(u * u, p, u);
-  return fabsf(u) < 0.25f ? p : __expf(u) - 1.f;
-}
-
-// cos(t) - 1 and sin(t) as rot_t (sweep_common.cuh) gives them: the Taylor
-// series below 1/2, rot_t beyond (not inlined: the argument reduction is
-// hundreds of instructions).
-__device__ __noinline__ float2 rot_far(float t) {
-  float c1, s1;
-  rot_t(t, &c1, &s1);
-  return make_float2(c1, s1);
-}
-__device__ __forceinline__ float2 rot_near(float t) {
-  const float q = t * t;
-  float c = fmaf(q, 1.f / 40320.f, -1.f / 720.f);
-  c = fmaf(q, c, 1.f / 24.f);
-  c = fmaf(q, c, -0.5f);
-  float s = fmaf(q, 1.f / 362880.f, -1.f / 5040.f);
-  s = fmaf(q, s, 1.f / 120.f);
-  s = fmaf(q, s, -1.f / 6.f);
-  return make_float2(q * c, fmaf(t * q, s, t));
-}
-
 template <bool IMAG, int H, int L>
 __global__ void __launch_bounds__(res_threads(H), 1) k_resident(const res_args a) {
   constexpr int NF = kResPlanes, NT = res_threads(H), NW = NT / 32;
@@ -382,12 +334,7 @@ __global__ void __launch_bounds__(res_threads(H), 1) k_resident(const res_args a
         // sweep adds it to the change of its points)
         const float2 s = make_float2(fmaf(sm1, p.x, p.x), fmaf(sm1, p.y, p.y));
         const float t = a.dt * fmaf(gs, fmaf(s.x, s.x, s.y * s.y), fmaf(a.hgam2 * x, x, vy));
-        const float2 k = fabsf(t) < 0.5f ? rot_near(t) : rot_far(t);
-        const float2 dl = make_float2(fmaf(k.x, s.x, k.y * s.y), fmaf(k.x, s.y, -(k.y * s.x)));
-        const float2 w = make_float2(__fadd_rn(s.x, dl.x), __fadd_rn(s.y, dl.y));
-        A[at] = w;
-        D[at] = make_float2(__fsub_rn(dl.x, __fsub_rn(w.x, s.x)),
-                                    __fsub_rn(dl.y, __fsub_rn(w.y, s.y)));
+        rotate_split(s, t, &A[at], &D[at]);
       }
     };
     ulonglong2 v[KH];

@@ -71,5 +71,14 @@ cudaError_t launch_res_tables(float2* tab, int nlines, int iters, const axis_coe
 
 // Does a step of this mode of the context run in the on-chip stepper?
 bool ctx_resident(const rotgp_ctx* c, bool imag);
+// Points over which a line carry of the context stays above the rounding of
+// the exact partition solve (hybrid.cuh).
+int ctx_carry_reach(const rotgp_ctx* c);
+// (batch_kernel.cu; reach: ctx_carry_reach of every instance)
+struct ctx_view;
+struct batch_dev;
+cudaError_t batch_kernel_run(batch_dev** d, const ctx_view* v, const int* reach, int count,
+                             const int* active, int nact, long long nsteps, bool imag,
+                             cudaStream_t s);
 
 }  // namespace rotgp

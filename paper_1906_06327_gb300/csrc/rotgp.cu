@@ -20,6 +20,7 @@
 #include "dsteps.cuh"
 #include "observe.cuh"
 #include "resident.cuh"
+#include "tails.cuh"
 #include "tma.cuh"
 
 using namespace rotgp;
@@ -125,10 +126,13 @@ struct rotgp_ctx {
   bool user_plan = false;
   bool res_ok[2] = {false, false};
   res_plan rplan[2];
-  float2* rtab[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};  // [axis][mode]
+  // weights of the two-tail line solve [axis][mode], and the tiles of its
+  // sweeps (tails.cu; blocks 0: not served)
+  float2* rtab[3][2] = {{nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr}};
+  tail_shape tails[3][2];
   float2* rsched[2] = {nullptr, nullptr};  // tables of kResSchedule steps, per axis
   unsigned long long* xbuf = nullptr;      // two exchange planes,
-  res_sync* rsync = nullptr;               // ... the exchange words (and rtab) behind them
+  res_sync* rsync = nullptr;               // ... the exchange words behind them
   // imaginary time in complex double (dsteps.cu), while the plan is the
   // default one: weights per axis, points per lane of the rows, own points of
   // the columns' segments (0: not served); dsync for whole blocks of 2D steps
@@ -689,7 +693,7 @@ int axis_tables(rotgp_ctx* c, int a, int mode) {
   Timed t(c, K_TABLES);
   cudaError_t e = launch_tables(c->fp64, ap.table[mode], ap.tableT[mode], ap.nlines, c->lt,
                                 ap.co[mode], c->stream);
-  if (e == cudaSuccess && a < 2 && c->rtab[a][mode]) {
+  if (e == cudaSuccess && c->rtab[a][mode]) {
     const res_omegas one{{1.0}};
     e = launch_res_tables(c->rtab[a][mode], ap.nlines, c->lt, ap.co[mode], one, 1, c->stream);
   }
@@ -712,8 +716,23 @@ void double_plan(rotgp_ctx* c) {
   }
 }
 
+// Tiles of the two-tail sweeps for the present halo.
+void tails_plan(rotgp_ctx* c) {
+  for (int a = 0; a < c->grid.dim; ++a)
+    for (int m = 0; m < 2; ++m) {
+      tail_shape& t = c->tails[a][m];
+      t = tail_shape{};
+      const AxisPlan& ap = c->axis[a];
+      if (!c->rtab[a][m] || !c->chunk_ok) continue;
+      if (!tail_plan(a, ap.len, c->nx, ap.lines, c->halo, m == 1, (size_t)c->smem_optin - 2048, &t) ||
+          (a == c->grid.dim - 1 && (size_t)t.blocks > c->partial_doubles))
+        t = tail_shape{};
+    }
+}
+
 int build_tables(rotgp_ctx* c) {
   double_plan(c);
+  tails_plan(c);
   for (int a = 0; a < c->grid.dim; ++a) {
     c->axis[a].wtab_fresh = false;
     for (int mode = 0; mode < 2; ++mode) {
@@ -920,7 +939,64 @@ int xy_pass(rotgp_ctx* c, bool imag) {
   return ROTGP_OK;
 }
 
+// Does this sweep run in the two-tail tiles?  Complex float, while no form or
+// shape is asked for: lines with a halo above the chunked TMA sweeps' 16
+// points (a 4096^2 step with halo 24 takes 174 us there, 311 in the exact
+// partition solve), and rows that are not 16-byte multiples, which the TMA
+// sweeps cannot read (255 x 256 x 128 167 us against 194 in imaginary time, 171
+// against 233 in real time; 65 x 49 x 33 27 against 36).  On even rows the TMA
+// sweeps are the faster ones (256 x 256 x 128 67 us).
+bool tail_sweep(const rotgp_ctx* c, int axis, bool imag) {
+  return !c->fp64 && !c->user_plan && c->tails[axis][imag ? 1 : 0].blocks > 0 &&
+         (c->halo > 16 || c->nx % 2 != 0);
+}
+
+int tail_step(rotgp_ctx* c, int axis, bool imag, bool last) {
+  const int mode = imag ? 1 : 0;
+  const AxisPlan& ap = c->axis[axis];
+  tail_args a{};
+  a.in = static_cast<const float2*>(c->psi[c->cur]);
+  a.out = static_cast<float2*>(c->psi[1 - c->cur]);
+  a.tab = c->rtab[axis][mode];
+  a.tlines = ap.nlines;
+  a.nx = c->nx;
+  a.ny = c->ny;
+  a.axis = axis;
+  a.len = ap.len;
+  a.H = std::max(1, c->halo - 2);
+  a.sh = c->tails[axis][mode];
+  a.lines = ap.lines;
+  a.dt = (float)c->phys.dt;
+  a.g = (float)c->phys.g;
+  a.hgam2 = (float)(0.5 * c->phys.gamma * c->phys.gamma);
+  a.hnu2 = (float)(0.5 * c->phys.nu * c->phys.nu);
+  a.hlam2 = c->grid.dim == 3 ? (float)(0.5 * c->phys.lambda * c->phys.lambda) : 0.f;
+  a.x0 = (float)c->x0;
+  a.hx = (float)c->grid.h[0];
+  a.y0 = c->y0;
+  a.hy = c->grid.h[1];
+  a.z0 = c->z0;
+  a.hz = c->grid.dim == 3 ? c->grid.h[2] : 0.0;
+  a.scale = c->d_scale();
+  a.vol = c->vol;
+  a.imag = mode;
+  a.partials = c->partials;
+  a.counter = c->counter;
+  a.scale_out = c->d_scale();
+  a.norm_out = c->d_norm();
+  a.flags = c->d_flags();
+  cudaError_t e;
+  {
+    Timed t(c, axis == 0 ? K_SWEEP_X : (axis == 1 ? K_SWEEP_Y : K_SWEEP_Z));
+    e = axis == 0 ? launch_tail_x(imag, a, c->stream) : launch_tail_s(last, a, c->stream);
+  }
+  if (e != cudaSuccess) return cuda_fail(c, e, "two-tail sweep launch");
+  c->cur = 1 - c->cur;
+  return ROTGP_OK;
+}
+
 int sweep(rotgp_ctx* c, int axis, bool imag, bool last) {
+  if (tail_sweep(c, axis, imag)) return tail_step(c, axis, imag, last);
   const int mode = imag ? 1 : 0;
   AxisPlan ap = c->axis[axis];
   if (!imag && !c->fp64 && ap.sh.V == 1 && (ap.sh.C == 8 || ap.sh.C == 16) && ap.rt.set &&
@@ -959,6 +1035,7 @@ int sweep(rotgp_ctx* c, int axis, bool imag, bool last) {
   cudaError_t e;
   if (ap.use_hybrid) {
     // exact partition solve, every precision and mode (H1 fused into x)
+    a.halo = ctx_carry_reach(c);
     a.coef_mode = axis == 0 ? 2 : (axis == 1 ? 1 : 0);
     a.stride = axis == 1 ? (long long)c->nx : (long long)c->nx * c->ny;
     a.outer = axis == 1 ? (long long)c->nx * c->ny : (long long)c->nx;
@@ -1198,6 +1275,12 @@ int encode_state_map(CUtensorMap* map, void* base, int nx, int ny, int nz, unsig
 int ctx_buffer(const rotgp_ctx* c) { return c->cur; }
 void ctx_set_buffer(rotgp_ctx* c, int cur) { c->cur = cur; }
 long long ctx_steps(const rotgp_ctx* c) { return c->steps; }
+int ctx_carry_reach(const rotgp_ctx* c) {
+  // a thousandth of the rounding of float, of double
+  const double tol = c->fp64 ? 1e-19 : 1e-10;
+  if (!(c->decay < 1.0)) return 1 << 20;
+  return c->decay <= 1e-6 ? 4 : (int)std::ceil(std::log(tol) / std::log(c->decay)) + 1;
+}
 bool ctx_resident(const rotgp_ctx* c, bool imag) {
   return resident(c, imag) || double_blocks(c, imag);
 }
@@ -1424,6 +1507,16 @@ int rotgp_create(const rotgp_grid* grid, const rotgp_phys* phys, int precision, 
     if (last.hyb_ok)
       pd = std::max(pd, (size_t)(hybrid_groups(la, last.lines, c->nx) * 8));
   }
+  if (!c->fp64 && c->chunk_ok) {
+    // ... of the last axis' two-tail tiles
+    const AxisPlan& last = c->axis[grid->dim - 1];
+    for (int m = 0; m < 2; ++m) {
+      tail_shape t;
+      if (tail_plan(grid->dim - 1, last.len, c->nx, last.lines, c->halo, m == 1,
+                    (size_t)c->smem_optin - 2048, &t))
+        pd = std::max(pd, (size_t)t.blocks);
+    }
+  }
   if (c->fp64) {
     // ... of the last axis' segments in complex double
     const AxisPlan& last = c->axis[grid->dim - 1];
@@ -1487,23 +1580,20 @@ int rotgp_create(const rotgp_grid* grid, const rotgp_phys* phys, int precision, 
       c->res_ok[m] = res_make_plan(c->nx, c->ny, c->halo, m == 1, c->sm_count,
                                    (size_t)c->smem_optin - 4096, &c->rplan[m]);
     if (c->res_ok[0] || c->res_ok[1]) {
-      // one allocation: exchange planes, exchange words, the lines' weights
+      // exchange planes with the exchange words behind them
       const size_t planes = 4 * (size_t)c->sites * sizeof(unsigned long long);
-      const size_t sync = (sizeof(res_sync) + 255) & ~(size_t)255;
-      const size_t wx = (size_t)kResPlanes * c->ny, wy = (size_t)kResPlanes * c->nx;
-      rc = dev_alloc(c, (void**)&c->xbuf, planes + sync + 2 * (wx + wy) * sizeof(float2));
+      rc = dev_alloc(c, (void**)&c->xbuf, planes + sizeof(res_sync));
       if (!rc) {
         c->rsync = reinterpret_cast<res_sync*>(reinterpret_cast<char*>(c->xbuf) + planes);
-        float2* w = reinterpret_cast<float2*>(reinterpret_cast<char*>(c->rsync) + sync);
-        for (int m = 0; m < 2; ++m) {
-          c->rtab[0][m] = w + m * (wx + wy);
-          c->rtab[1][m] = c->rtab[0][m] + wx;
-        }
-        e = cudaMemsetAsync(c->xbuf, 0, planes + sync, c->stream);
+        e = cudaMemsetAsync(c->xbuf, 0, planes + sizeof(res_sync), c->stream);
         if (e != cudaSuccess) rc = cuda_fail(c, e, "initialise buffers");
       }
     }
   }
+  for (int a = 0; a < grid->dim && !rc && !c->fp64 && c->chunk_ok; ++a)
+    for (int m = 0; m < 2 && !rc; ++m)
+      rc = dev_alloc(c, (void**)&c->rtab[a][m],
+                     (size_t)kResPlanes * c->axis[a].nlines * sizeof(float2));
   if (!rc && c->fp64 && c->chunk_ok && c->halo <= kDPow) {
     size_t lines = 0;
     for (int a = 0; a < grid->dim; ++a) lines += c->axis[a].nlines;
@@ -2055,12 +2145,12 @@ int rotgp_autotune(rotgp_ctx* c, int steps, int* choice) {
     }
     ap.lsegs = best_s;
   }
-  // and the on-chip 2D stepper or the complex-double kernels, which take no
-  // form or shape
+  // and the default plan where it has kernels that take no form or shape
   if (e == cudaSuccess && !rc) {
     c->user_plan = false;
     float ms = 0;
-    if ((resident(c, true) || double_steps(c, true)) && time_current(&ms) && ms < best_ms)
+    if ((resident(c, true) || double_steps(c, true) || tail_sweep(c, 0, true)) &&
+        time_current(&ms) && ms < best_ms)
       best = 0;
     else
       c->user_plan = true;
