@@ -232,11 +232,10 @@ int rotgp_info(const rotgp_ctx* ctx, rotgp_solver_info* out);
  * block, taking 32-line units round-robin) and
  * segments each line is split into (clamped to the number of chunks).
  * The one-line-per-thread TMA forms (chunk 8 or 16) solve the unfolded
- * system psi' = 2 A^-1 psi - psi and serve imaginary-time steps; real-time
- * steps of an axis so tuned run the default two-lines-per-thread form, whose
- * folded weights keep the CN map's norm to float rounding.  Changes speed only: every shape gives results
- * equal up to the truncation bound of the chunked line solver.  Used by the
- * autotuner.  On an axis in the exact partition solve (ROTGP_SOLVER_HYBRID)
+ * system psi' = 2 A^-1 psi - psi, in real time centred about psi so that its
+ * rounded weights keep the CN map's norm.  Changes speed only: every shape
+ * gives results equal up to the truncation bound of the chunked line solver.
+ * Used by the autotuner.  On an axis in the exact partition solve (ROTGP_SOLVER_HYBRID)
  * only `segments` applies: the number of CTAs (1, 2, 4 or 8, one cluster)
  * that share each line; results are equal up to rounding.
  * ROTGP_EINVAL for a shape that is not built or does not fit. */

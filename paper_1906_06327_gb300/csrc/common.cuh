@@ -52,7 +52,7 @@ __device__ __forceinline__ T abs2(cpx<T> a) { return a.x * a.x + a.y * a.y; }
 // stored as the difference the rounding is that many times smaller.
 // m2 = 2 m_p serves the unfolded form of the same solve (psi' = 2y - psi
 // with A y = psi): d_p = m2 psi_p + al d_{p-1}, z_p = d_p + be z_{p+1},
-// psi'_p = z_p - psi_p.
+// psi'_p = z_p - psi_p (real time: its centred form, k_sweep_s1t).
 // Entry 0 is all zero (the Dirichlet edge); entries past the table length
 // equal the last one (the Toeplitz fixed point).
 template <class T>
@@ -80,7 +80,8 @@ struct stream_args {
   void* out;
   const void* coef;   // coef5<T>[coefficient lines][lt + 1]
   // the same unfolded-form weights of complex float as three planes
-  // [m2, al, be][lt + 1][coefficient lines] (consecutive lines contiguous)
+  // [m2, al, be][lt + 1][coefficient lines] (consecutive lines contiguous);
+  // m2 - 2 in place of m2 in real time
   const float2* coefT;
   int tlines;         // coefficient lines
   int len;            // N: stored points per line
@@ -167,16 +168,6 @@ struct obs_args {
 enum { NQ = 14 };   // partial sums per block in the observables reduction (last: a max)
 enum { NOBS = 12 }; // norm, mu, E, mu_c, E_c, rms_x, rms_y, rms_z, rms_r, max, mu4, E4
 
-struct vort_args {
-  const void* psi;
-  int nx, ny, nz, dim, kplane;
-  double hx, hy, x0, y0;
-  double* partials;
-  unsigned int* counter;
-  double* moments;  // rx2, ry2
-  int* count;
-};
-
 // ---- launchers (one per translation unit group); return cudaGetLastError
 // Launch shape of one sweep, chosen on the host.
 struct sweep_shape {
@@ -191,7 +182,7 @@ struct sweep_shape {
 
 // tableT: the planes of stream_args::coefT (complex float only), or null
 cudaError_t launch_tables(bool fp64, void* table, void* tableT, int nlines, int lt,
-                          const axis_coef& co, cudaStream_t s);
+                          const axis_coef& co, bool imag, cudaStream_t s);
 // map: rows TMA map of the input buffer or null; omap: the swizzled
 // one-row-per-lane map of the output buffer (that form only) or null
 cudaError_t launch_sweep_x(bool fp64, bool imag, const stream_args& a, const sweep_shape& sh,
@@ -279,12 +270,6 @@ inline bool sweep_shape_built(bool fp64, int V, int C) {
   if (fp64) return V == 1 && (C == 16 || C == 64);
   return (V == 2 && (C == 8 || C == 16)) || (V == 1 && (C == 16 || C == 64));
 }
-cudaError_t launch_observables(bool fp64, const obs_args& a, int blocks, int threads,
-                               cudaStream_t s);
-cudaError_t launch_vortex_moments(bool fp64, const vort_args& a, int blocks, int threads,
-                                  cudaStream_t s);
-cudaError_t launch_vortex_count(bool fp64, const vort_args& a, int blocks, int threads,
-                                cudaStream_t s);
 cudaError_t launch_norm(bool fp64, const void* psi, long long nsites, double vol, int imag_scale,
                         double* partials, unsigned int* counter, double* scale_out,
                         double* norm_out, int* flags, int blocks, int threads, cudaStream_t s);
@@ -293,8 +278,6 @@ cudaError_t launch_init_analytic(bool fp64, void* psi, int nx, int ny, int nz, i
                                  double hz, int function, int phase_mode, const double* R,
                                  unsigned long long seed, double d_xy, double d_z,
                                  cudaStream_t s);
-cudaError_t launch_pack(bool fp64_store, bool fp64_src, const void* src, void* psi, int nx,
-                        int ny, int nz, int dim, double* scale, cudaStream_t s);
 cudaError_t launch_unpack(bool fp64_store, bool fp64_dst, const void* psi, void* dst, int nx,
                           int ny, int nz, int dim, const double* scale, cudaStream_t s);
 cudaError_t launch_set_scalar(double* p, double v, cudaStream_t s);
@@ -325,8 +308,10 @@ void ctx_get_view(const rotgp_ctx* c, ctx_view* v);
 struct batch_dev;
 void batch_kernel_free(batch_dev* d);
 bool batch_kernel_fits(const ctx_view* v, int count, size_t smem_limit, const char** why);
-cudaError_t batch_kernel_run(batch_dev** d, const ctx_view* v, int count, const int* active,
-                             int nact, long long nsteps, bool imag, cudaStream_t s);
+// (reach: ctx_carry_reach of every instance)
+cudaError_t batch_kernel_run(batch_dev** d, const ctx_view* v, const int* reach, int count,
+                             const int* active, int nact, long long nsteps, bool imag,
+                             cudaStream_t s);
 cudaError_t batch_kernel_flags(batch_dev* d, cudaStream_t s, int* flags);
 
 }  // namespace rotgp

@@ -74,11 +74,5 @@ bool ctx_resident(const rotgp_ctx* c, bool imag);
 // Points over which a line carry of the context stays above the rounding of
 // the exact partition solve (hybrid.cuh).
 int ctx_carry_reach(const rotgp_ctx* c);
-// (batch_kernel.cu; reach: ctx_carry_reach of every instance)
-struct ctx_view;
-struct batch_dev;
-cudaError_t batch_kernel_run(batch_dev** d, const ctx_view* v, const int* reach, int count,
-                             const int* active, int nact, long long nsteps, bool imag,
-                             cudaStream_t s);
 
 }  // namespace rotgp

@@ -51,15 +51,6 @@ struct AxisPlan {
   int len = 0;          // points per line
   int nseg = 1, seg_chunks = 1, warm = 1;
   sweep_shape sh{};
-  // real-time launch plan when sh is a one-line-per-lane TMA (unfolded)
-  // shape: that form rounds 2 A^-1 psi before subtracting psi, which doubles
-  // the effect of the rounded weights and drifts the real-time norm; real
-  // time keeps the folded two-lines-per-lane form
-  struct {
-    bool set = false;
-    int nseg = 1, seg_chunks = 1, warm = 1;
-    sweep_shape sh{};
-  } rt;
   // banded-inverse stencil (complex float): taps K, end rows B, weights [mode]
   bool stencil_ok = false;  // stencil form available for this axis
   bool use_stencil = false;
@@ -463,13 +454,6 @@ int plan_axes(rotgp_ctx* c) {
     const long long groups = (ap.lines + 32 * V - 1) / (32 * V);
     int rc = set_shape(c, a, V, C, R, 1, std::max<long long>(1, target / groups));
     if (rc) return rc == ROTGP_EINVAL ? fail(c, ROTGP_EUNSUPPORTED, "%s", c->err.c_str()) : rc;
-    // this folded plan also serves real-time steps whenever a one-line-per-
-    // lane TMA (unfolded) shape is chosen for the axis later
-    ap.rt.set = true;
-    ap.rt.nseg = ap.nseg;
-    ap.rt.seg_chunks = ap.seg_chunks;
-    ap.rt.warm = ap.warm;
-    ap.rt.sh = ap.sh;
     // banded-inverse stencil: complex float, even N_x (TMA rows of 16-byte
     // multiples; the separate x-stencil kernel also wants N_x % 4 == 0)
     int K = 0, B = 0;
@@ -692,7 +676,7 @@ int axis_tables(rotgp_ctx* c, int a, int mode) {
                           nlines_du(c, a));
   Timed t(c, K_TABLES);
   cudaError_t e = launch_tables(c->fp64, ap.table[mode], ap.tableT[mode], ap.nlines, c->lt,
-                                ap.co[mode], c->stream);
+                                ap.co[mode], mode == 1, c->stream);
   if (e == cudaSuccess && c->rtab[a][mode]) {
     const res_omegas one{{1.0}};
     e = launch_res_tables(c->rtab[a][mode], ap.nlines, c->lt, ap.co[mode], one, 1, c->stream);
@@ -945,7 +929,8 @@ int xy_pass(rotgp_ctx* c, bool imag) {
 // partition solve), and rows that are not 16-byte multiples, which the TMA
 // sweeps cannot read (255 x 256 x 128 167 us against 194 in imaginary time, 171
 // against 233 in real time; 65 x 49 x 33 27 against 36).  On even rows the TMA
-// sweeps are the faster ones (256 x 256 x 128 67 us).
+// sweeps are the faster ones (256 x 256 x 128 67 us in imaginary and 87 us in
+// real time, against 145 in tiles).
 bool tail_sweep(const rotgp_ctx* c, int axis, bool imag) {
   return !c->fp64 && !c->user_plan && c->tails[axis][imag ? 1 : 0].blocks > 0 &&
          (c->halo > 16 || c->nx % 2 != 0);
@@ -998,14 +983,7 @@ int tail_step(rotgp_ctx* c, int axis, bool imag, bool last) {
 int sweep(rotgp_ctx* c, int axis, bool imag, bool last) {
   if (tail_sweep(c, axis, imag)) return tail_step(c, axis, imag, last);
   const int mode = imag ? 1 : 0;
-  AxisPlan ap = c->axis[axis];
-  if (!imag && !c->fp64 && ap.sh.V == 1 && (ap.sh.C == 8 || ap.sh.C == 16) && ap.rt.set &&
-      (axis == 0 ? c->xmaps_ok && c->x_tma : c->smaps_ok)) {
-    ap.nseg = ap.rt.nseg;
-    ap.seg_chunks = ap.rt.seg_chunks;
-    ap.warm = ap.rt.warm;
-    ap.sh = ap.rt.sh;
-  }
+  const AxisPlan& ap = c->axis[axis];
   stream_args a{};
   a.in = c->psi[c->cur];
   a.out = c->psi[1 - c->cur];
@@ -1127,10 +1105,10 @@ int run_steps(rotgp_ctx* c, long long n, bool imag) {
     for (int a = 0; a < c->grid.dim; ++a) {
       int rc;
       // the stencil and fused forms serve imaginary time; real-time steps
-      // keep the folded Thomas form, whose near-unit diagonal factor is
-      // stored as its difference from 1 so that the rounded CN map stays
-      // unitary to ~1e-10 per sweep (the stencil's rounded central weight,
-      // close to 1 itself, would not)
+      // keep Thomas forms whose near-unit factors are stored as their
+      // difference from 1 or 2, so that the rounded CN map stays unitary to
+      // ~1e-10 per sweep (the stencil's rounded central weight, close to 1
+      // itself, would not)
       if (a == 0 && c->fuse_xy && imag) {
         rc = xy_pass(c, imag);
         ++a;  // the y sweep is part of the pass

@@ -28,8 +28,9 @@
 // k_sweep_s1t) use the same chunking with the unfolded solve of the same
 // system (A y = psi, psi' = 2y - psi: weights m2, al, be, no neighbour
 // points), TMA box loads and stores through R + 1 slots per warp, persistent
-// warps and programmatic launch; they serve imaginary time, while real time
-// keeps the folded form above (it holds the CN map's norm to rounding).
+// warps and programmatic launch; real time solves it in the centred form
+// (weight m2 - 2, see k_sweep_s1t), which holds the CN map's norm to rounding
+// as the folded form above does.
 #pragma once
 
 #include "common.cuh"

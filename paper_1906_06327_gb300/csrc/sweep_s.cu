@@ -37,7 +37,8 @@ template <class T>
 __device__ __forceinline__ cpx<T> dcast(dcx a) { return mk<T>((T)a.x, (T)a.y); }
 
 template <class T>
-__global__ void k_tables(coef5<T>* tab, float2* tabT, int nlines, int lt, axis_coef co) {
+__global__ void k_tables(coef5<T>* tab, float2* tabT, int nlines, int lt, axis_coef co,
+                         double m2_less) {
   const int l = blockIdx.x * blockDim.x + threadIdx.x;
   if (l >= nlines) return;
   const double u = co.u0 + (double)l * co.du;
@@ -49,6 +50,7 @@ __global__ void k_tables(coef5<T>* tab, float2* tabT, int nlines, int lt, axis_c
   const dcx kmt = dsub(kap, tau), kpt{kap.x + tau.x, kap.y + tau.y};
   coef5<T>* t = tab + (size_t)l * (lt + 1);
   t[0].a0 = t[0].am = t[0].ap = t[0].al = t[0].be = t[0].m2 = zero<T>();
+  if (tabT) tabT[l] = make_float2(0.f, 0.f);
   dcx c{0.0, 0.0};
   for (int p = 1; p <= lt; ++p) {
     const dcx m = dinv(dsub(a0, dmul(am, c)));
@@ -61,12 +63,13 @@ __global__ void k_tables(coef5<T>* tab, float2* tabT, int nlines, int lt, axis_c
     t[p].al = dcast<T>({-mam.x, -mam.y});
     t[p].be = dcast<T>({-c.x, -c.y});
     t[p].m2 = dcast<T>({2.0 * m.x, 2.0 * m.y});
+    if (tabT)
+      tabT[(size_t)p * nlines + l] = make_float2((float)(2.0 * m.x - m2_less), (float)(2.0 * m.y));
   }
   if (tabT) {
     const size_t P = (size_t)(lt + 1) * nlines;
     for (int p = 0; p <= lt; ++p) {
       const size_t i = (size_t)p * nlines + l;
-      tabT[i] = make_float2((float)t[p].m2.x, (float)t[p].m2.y);
       tabT[P + i] = make_float2((float)t[p].al.x, (float)t[p].al.y);
       tabT[2 * P + i] = make_float2((float)t[p].be.x, (float)t[p].be.y);
     }
@@ -362,14 +365,17 @@ __global__ void __launch_bounds__(128) k_sweep_strided2(const stream_args a) {
 
 // --------------------------------------------------------------- launchers
 cudaError_t launch_tables(bool fp64, void* table, void* tableT, int nlines, int lt,
-                          const axis_coef& co, cudaStream_t s) {
-  const int threads = 128, blocks = (nlines + threads - 1) / threads;
+                          const axis_coef& co, bool imag, cudaStream_t s) {
+  // a warp per block: the recursion is a chain of double operations, and a
+  // warp has a scheduler's double pipe to itself
+  const int threads = 32, blocks = (nlines + threads - 1) / threads;
   if (fp64)
     k_tables<double><<<blocks, threads, 0, s>>>(static_cast<coef5<double>*>(table), nullptr,
-                                                nlines, lt, co);
+                                                nlines, lt, co, 0.0);
   else
     k_tables<float><<<blocks, threads, 0, s>>>(static_cast<coef5<float>*>(table),
-                                               static_cast<float2*>(tableT), nlines, lt, co);
+                                               static_cast<float2*>(tableT), nlines, lt, co,
+                                               imag ? 0.0 : 2.0);
   return cudaGetLastError();
 }
 
@@ -510,7 +516,16 @@ static cudaError_t dispatch_s2(bool reduce, const stream_args& a, const sweep_sh
 // forward sweep, the chunk being back-substituted, and one more whose store
 // may still be reading shared memory.  Arithmetic on the interleaved
 // (re, im) layout with packed FP32x2 (cacc form, sweep_common.cuh).
-template <int C, bool REDUCE, int RING, int AX>
+//
+// CEN (real time): the centred form of the same solve, whose weights are all
+// of the order of kappa (mc = m2 - 2 in the first plane): t_p = d_p - 2 psi_p =
+// mc psi_p + al d_{p-1}, psi'_p = psi_p + (t_p + be z_{p+1}).  The plain form
+// doubles the rounding of m2 every step, which moves the real-time norm by
+// 2e-4 per time unit; this one keeps it as the folded two-lines-per-lane
+// sweeps do (1e-9 per step), at two more operations a point instead of four
+// more complex products (GB300, 256 x 256 x 128 real-time step 128 us in the
+// folded sweeps, 87.5 in these).
+template <int C, bool REDUCE, int RING, int AX, bool CEN>
 __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_s1t(const __grid_constant__ CUtensorMap map,
                                                    const __grid_constant__ CUtensorMap omap,
                                                    const stream_args a) {
@@ -579,6 +594,10 @@ __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_s1t(const __grid_c
       const float2 A = __ffma2_rn(br, z, dp), B = __fmul2_rn(bi, z);
       return make_float2(A.x - B.y, A.y + B.x);
     };
+    // CEN: the value from psi and the small part t or t + be z
+    auto twice = [](float2 psi, float2 t) -> float2 {
+      return __ffma2_rn(make_float2(2.f, 2.f), psi, t);
+    };
     auto coords = [&](int q, int& c1, int& c2) {
       c1 = AX == 1 ? q * C : gt;
       c2 = AX == 1 ? gt : q * C;
@@ -617,8 +636,10 @@ __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_s1t(const __grid_c
         if (p0 >= lt && p0 + C <= N) {
 #pragma unroll
           for (int r = 0; r < C; ++r) {
-            d = fwd(M2R, M2I, ALR, ALI, sp[r * 32], d);
+            const float2 v = sp[r * 32];
+            d = fwd(M2R, M2I, ALR, ALI, v, d);
             cur[r] = d;
+            if (CEN) d = twice(v, d);
           }
         } else {
           float2 km[C], kl[C];
@@ -628,8 +649,10 @@ __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_s1t(const __grid_c
             float2 mr, mi, lr, li;
             wsplit(km[r], mr, mi);
             wsplit(kl[r], lr, li);
-            d = fwd(mr, mi, lr, li, sp[r * 32], d);
+            const float2 v = sp[r * 32];
+            d = fwd(mr, mi, lr, li, v, d);
             cur[r] = d;
+            if (CEN) d = twice(v, d);
           }
         }
       }
@@ -639,9 +662,13 @@ __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_s1t(const __grid_c
         float2 z = make_float2(0.f, 0.f);
         if (q < qb) {
           const int p0 = q * C;
+          const float2* sn = ring + (size_t)sq * SLOT + lane;
           if (p0 >= lt && p0 + C <= N) {
 #pragma unroll
-            for (int h = C - 1; h >= 0; --h) z = bstep(BER, BEI, z, cur[h]);
+            for (int h = C - 1; h >= 0; --h) {
+              z = bstep(BER, BEI, z, cur[h]);
+              if (CEN) z = twice(sn[h * 32], z);
+            }
           } else {
             float2 kb[C];
             table_be<C>(tab, tl, lt, li, p0, pol_last, kb);
@@ -651,6 +678,7 @@ __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_s1t(const __grid_c
                 float2 br, bi;
                 wsplit(kb[h], br, bi);
                 z = bstep(br, bi, z, cur[h]);
+                if (CEN) z = twice(sn[h * 32], z);
               }
           }
         }
@@ -662,7 +690,9 @@ __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_s1t(const __grid_c
 #pragma unroll
           for (int r = C - 1; r >= 0; --r) {
             z = bstep(BER, BEI, z, prv[r]);
-            const float2 o = __ffma2_rn(NEG1, sp[r * 32], z);
+            const float2 v = sp[r * 32];
+            const float2 o = CEN ? __fadd2_rn(v, z) : __ffma2_rn(NEG1, v, z);
+            if (CEN) z = twice(v, z);
             sp[r * 32] = o;
             if (REDUCE) n2 = __ffma2_rn(o, o, n2);
           }
@@ -675,7 +705,9 @@ __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_s1t(const __grid_c
               float2 br, bi;
               wsplit(kb[r], br, bi);
               z = bstep(br, bi, z, prv[r]);
-              const float2 o = __ffma2_rn(NEG1, sp[r * 32], z);
+              const float2 v = sp[r * 32];
+              const float2 o = CEN ? __fadd2_rn(v, z) : __ffma2_rn(NEG1, v, z);
+              if (CEN) z = twice(v, z);
               sp[r * 32] = o;
               if (REDUCE) n2 = __ffma2_rn(o, o, n2);
             }
@@ -732,7 +764,8 @@ static cudaError_t dispatch_s1t(bool reduce, const stream_args& a, const sweep_s
                                 const void* map, const void* omap, cudaStream_t s) {
   const CUtensorMap& m = *static_cast<const CUtensorMap*>(map);
   const CUtensorMap& om = *static_cast<const CUtensorMap*>(omap);
-  auto fn = reduce ? k_sweep_s1t<C, true, R, AX> : k_sweep_s1t<C, false, R, AX>;
+  auto fn = a.imag ? (reduce ? k_sweep_s1t<C, true, R, AX, false> : k_sweep_s1t<C, false, R, AX, false>)
+                   : (reduce ? k_sweep_s1t<C, true, R, AX, true> : k_sweep_s1t<C, false, R, AX, true>);
   cudaError_t e = allow_smem((const void*)fn);
   if (e != cudaSuccess) return e;
   const long long units = (long long)((a.nx + 31) / 32) * (a.nlines / a.nx) * a.nseg;

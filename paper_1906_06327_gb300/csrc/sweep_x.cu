@@ -10,7 +10,7 @@
 // 16-byte shared loads (conflict-free) and the results go back through the
 // same slot for coalesced stores.  The solver and the ring are described in
 // sweep_common.cuh.
-#include "sweep_common.cuh"
+#include "tail_solve.cuh"
 #include "tma.cuh"
 
 namespace rotgp {
@@ -564,6 +564,11 @@ __global__ void __launch_bounds__(128) k_sweep_x2(const __grid_constant__ CUtens
 // SM with all the registers it wants (166); capped at 144 so that 14 warps
 // fit (one wave of units on the 512 x 512 x 128 state) it measured slower
 // on GB300 (141 against 114 us per sweep).
+//
+// Real time: the centred form of k_sweep_s1t (CEN there), the slot keeping the
+// advanced point rounded, and two more slots per warp, one per chunk in
+// flight, what that rounding left out, which joins the change of the point
+// before the point itself is added (see hpt in sweep_common.cuh).
 template <int C, bool IMAG, int RING>
 __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_x1t(const __grid_constant__ CUtensorMap map,
                                                    const __grid_constant__ CUtensorMap omap,
@@ -572,18 +577,20 @@ __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_x1t(const __grid_c
   constexpr int ROWS = 32;
   constexpr int U = C / 2;            // 16-byte units per row
   constexpr int SLOT = ROWS * C;      // float2 per slot (2 or 4 KB)
+  constexpr int WARP = (NS + (IMAG ? 0 : 2)) * SLOT;  // float2 per warp
   static_assert((C == 8 || C == 16) && (SLOT * 8) % 1024 == 0 && NS <= 8, "TMA slots");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bars[16 * 8];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   if (a.ring != RING || blockDim.x > (C == 8 ? 512u : 256u) ||
-      dynamic_smem_bytes() < (blockDim.x >> 5) * (unsigned)(NS * SLOT * 8) + 1024u) {
+      dynamic_smem_bytes() < (blockDim.x >> 5) * (unsigned)(WARP * 8) + 1024u) {
     if (threadIdx.x == 0) atomicOr(a.flags, 2);
     return;
   }
   // swizzled boxes repeat every 1024 bytes of shared address: align to it
   unsigned char* sbase = smem_raw + ((1024 - (smem_addr(smem_raw) & 1023)) & 1023);
-  float2* ring = reinterpret_cast<float2*>(sbase) + (size_t)wib * NS * SLOT;
+  float2* ring = reinterpret_cast<float2*>(sbase) + (size_t)wib * WARP;
+  float2* rest = ring + NS * SLOT + lane;  // real time: [chunk parity][point][lane]
   uint64_t* bar = bars + wib * 8;
   const long long nrows = a.nlines;
   const long long ngroups = (nrows + ROWS - 1) / ROWS;
@@ -628,18 +635,17 @@ __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_x1t(const __grid_c
     const float sc = (float)(*a.scale), hg2 = (float)a.hgam2, dt = (float)a.dt, gg = (float)a.g;
     const float xs = (float)a.x0, hx = (float)a.hx;
     const float2 SC = make_float2(sc, sc);
-    auto h1 = [&](float2 v, int p) -> float2 {
+    // real time: the point scaled and advanced, rounded, and the rest
+    auto h1 = [&](float2 v, int p, float2* rs) -> float2 {
       v = __fmul2_rn(SC, v);
       const float x = fmaf((float)p, hx, xs);
       const float en = fmaf(gg, fmaf(v.x, v.x, v.y * v.y), fmaf(hg2 * x, x, vyz));
-      if (IMAG) {
-        const float f = __expf(-dt * en);
-        return __fmul2_rn(make_float2(f, f), v);
-      } else {
-        float c1, s1;
-        rot_t(dt * en, &c1, &s1);
-        return rotate_f(v, c1, s1);
-      }
+      float2 w;
+      rotate_split(v, dt * en, &w, rs);
+      return w;
+    };
+    auto twice = [](float2 psi, float2 t) -> float2 {
+      return __ffma2_rn(make_float2(2.f, 2.f), psi, t);
     };
     // imaginary time: the factor sc exp(-dt (V + g sc^2 |v|^2)) of a raw
     // point v as one base-2 exponential of a quadratic in x and |v|^2, the
@@ -708,8 +714,9 @@ __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_x1t(const __grid_c
             w[2 * u] = h1i(make_float2(t.x, t.y), fmaf((float)(2 * u), hx, xp0));
             w[2 * u + 1] = h1i(make_float2(t.z, t.w), fmaf((float)(2 * u + 1), hx, xp0));
           } else {
-            w[2 * u] = h1(make_float2(t.x, t.y), p0 + 2 * u);
-            w[2 * u + 1] = h1(make_float2(t.z, t.w), p0 + 2 * u + 1);
+            float2* rs = rest + (q & 1) * SLOT + 2 * u * 32;
+            w[2 * u] = h1(make_float2(t.x, t.y), p0 + 2 * u, rs);
+            w[2 * u + 1] = h1(make_float2(t.z, t.w), p0 + 2 * u + 1, rs + 32);
           }
         }
         if (p0 >= lt && p0 + C <= N) {
@@ -717,6 +724,7 @@ __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_x1t(const __grid_c
           for (int r = 0; r < C; ++r) {
             d = fwd(M2R, M2I, ALR, ALI, w[r], d);
             cur[r] = d;
+            if (!IMAG) d = twice(w[r], d);
           }
         } else {
           float2 km[C], kl[C];
@@ -728,6 +736,7 @@ __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_x1t(const __grid_c
             wsplit(kl[r], lr, li);
             d = fwd(mr, mi, lr, li, w[r], d);
             cur[r] = d;
+            if (!IMAG) d = twice(w[r], d);
           }
         }
         // keep the H1-advanced points for the back substitution
@@ -743,28 +752,51 @@ __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_x1t(const __grid_c
           const int p0 = q * C;
           if (p0 >= lt && p0 + C <= N) {
 #pragma unroll
-            for (int h = C - 1; h >= 0; --h) z = bstep(BER, BEI, z, cur[h]);
+            for (int u = U - 1; u >= 0; --u) {
+              float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+              if (!IMAG) t = *unit(sq, u);
+              z = bstep(BER, BEI, z, cur[2 * u + 1]);
+              if (!IMAG) z = twice(make_float2(t.z, t.w), z);
+              z = bstep(BER, BEI, z, cur[2 * u]);
+              if (!IMAG) z = twice(make_float2(t.x, t.y), z);
+            }
           } else {
             float2 kb[C];
             table_be<C>(tab, tl, lt, li, p0, pol_last, kb);
 #pragma unroll
-            for (int h = C - 1; h >= 0; --h)
-              if (p0 + h < N) {
+            for (int u = U - 1; u >= 0; --u) {
+              float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+              if (!IMAG) t = *unit(sq, u);
+#pragma unroll
+              for (int e = 1; e >= 0; --e) {
+                const int h = 2 * u + e;
+                if (p0 + h >= N) continue;
                 float2 br, bi;
                 wsplit(kb[h], br, bi);
                 z = bstep(br, bi, z, cur[h]);
+                if (!IMAG) z = twice(e ? make_float2(t.z, t.w) : make_float2(t.x, t.y), z);
               }
+            }
           }
         }
         const int p0 = qq * C;
+        // the result of a point from psi (advanced) and z, which becomes the
+        // value of the recurrence
+        const float2* rq = rest + (qq & 1) * SLOT;
+        auto result = [&](float2 psi, int r) -> float2 {
+          if (IMAG) return __ffma2_rn(NEG1, psi, z);
+          const float2 o = __fadd2_rn(psi, __fadd2_rn(rq[r * 32], z));
+          z = twice(psi, z);
+          return o;
+        };
         if (p0 >= lt && p0 + C <= N) {
 #pragma unroll
           for (int u = U - 1; u >= 0; --u) {
             const float4 t = *unit(sp, u);
             z = bstep(BER, BEI, z, prv[2 * u + 1]);
-            const float2 o1 = __ffma2_rn(NEG1, make_float2(t.z, t.w), z);
+            const float2 o1 = result(make_float2(t.z, t.w), 2 * u + 1);
             z = bstep(BER, BEI, z, prv[2 * u]);
-            const float2 o0 = __ffma2_rn(NEG1, make_float2(t.x, t.y), z);
+            const float2 o0 = result(make_float2(t.x, t.y), 2 * u);
             *unit(sp, u) = make_float4(o0.x, o0.y, o1.x, o1.y);
           }
         } else {
@@ -782,7 +814,7 @@ __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_x1t(const __grid_c
                 wsplit(kb[r], br, bi);
                 z = bstep(br, bi, z, prv[r]);
               }
-              o[e] = __ffma2_rn(NEG1, e ? make_float2(t.z, t.w) : make_float2(t.x, t.y), z);
+              o[e] = result(e ? make_float2(t.z, t.w) : make_float2(t.x, t.y), r);
             }
             *unit(sp, u) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
           }
@@ -826,7 +858,9 @@ __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_x1t(const __grid_c
   if (lane == 0) bulk_wait_all();
 }
 
-size_t x1t_smem_per_warp(int C, int R) { return (size_t)(R + 1) * 32 * C * 8; }
+size_t x1t_smem_per_warp(int C, int R, bool imag) {
+  return (size_t)(R + (imag ? 1 : 3)) * 32 * C * 8;
+}
 
 template <int C, int R>
 static cudaError_t dispatch_x1t(bool imag, const stream_args& a, const sweep_shape& sh,
@@ -839,10 +873,10 @@ static cudaError_t dispatch_x1t(bool imag, const stream_args& a, const sweep_sha
   const long long units = (a.nlines + 31) / 32 * a.nseg;
   int W = 1;
   unsigned blocks = 0;
-  e = resident_grid((const void*)fn, units, x1t_smem_per_warp(C, R), 1024, C == 8 ? 16 : 8, &W,
+  e = resident_grid((const void*)fn, units, x1t_smem_per_warp(C, R, imag), 1024, C == 8 ? 16 : 8, &W,
                     &blocks);
   if (e != cudaSuccess) return e;
-  return launch_programmatic(fn, blocks, 32 * W, x1t_smem_per_warp(C, R) * W + 1024, s, m, om, a);
+  return launch_programmatic(fn, blocks, 32 * W, x1t_smem_per_warp(C, R, imag) * W + 1024, s, m, om, a);
 }
 
 template <int C, int R>
