@@ -153,18 +153,6 @@ struct tile_args {
   int* flags;            // bit 0 non-finite norm, bit 2 TMA wait timed out
 };
 
-struct obs_args {
-  const void* psi;
-  int nx, ny, nz, dim;
-  double hx, hy, hz, x0, y0, z0;
-  double hgam2, hnu2, hlam2, g, omega;
-  const double* scale;
-  int zchunk;          // z planes per work item (tiles of 32 x 8 columns)
-  double* partials;
-  unsigned int* counter;
-  double* result;  // NOBS doubles
-};
-
 enum { NQ = 14 };   // partial sums per block in the observables reduction (last: a max)
 enum { NOBS = 12 }; // norm, mu, E, mu_c, E_c, rms_x, rms_y, rms_z, rms_r, max, mu4, E4
 
