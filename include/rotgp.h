@@ -233,7 +233,8 @@ int rotgp_info(const rotgp_ctx* ctx, rotgp_solver_info* out);
  * segments each line is split into (clamped to the number of chunks).
  * The one-line-per-thread TMA forms (chunk 8 or 16) solve the unfolded
  * system psi' = 2 A^-1 psi - psi, in real time centred about psi so that its
- * rounded weights keep the CN map's norm.  Changes speed only: every shape
+ * rounded weights keep the CN map's norm; an axis with Delta / (4 h^2) above
+ * 0.005 runs its real-time steps in the default two-lines-per-thread form.  Changes speed only: every shape
  * gives results equal up to the truncation bound of the chunked line solver.
  * Used by the autotuner.  On an axis in the exact partition solve (ROTGP_SOLVER_HYBRID)
  * only `segments` applies: the number of CTAs (1, 2, 4 or 8, one cluster)

@@ -51,6 +51,13 @@ struct AxisPlan {
   int len = 0;          // points per line
   int nseg = 1, seg_chunks = 1, warm = 1;
   sweep_shape sh{};
+  // the folded plan of real-time steps whose kappa is too large for the centred
+  // TMA sweeps (see centred_ok)
+  struct {
+    bool set = false;
+    int nseg = 1, seg_chunks = 1, warm = 1;
+    sweep_shape sh{};
+  } rt;
   // banded-inverse stencil (complex float): taps K, end rows B, weights [mode]
   bool stencil_ok = false;  // stencil form available for this axis
   bool use_stencil = false;
@@ -454,6 +461,11 @@ int plan_axes(rotgp_ctx* c) {
     const long long groups = (ap.lines + 32 * V - 1) / (32 * V);
     int rc = set_shape(c, a, V, C, R, 1, std::max<long long>(1, target / groups));
     if (rc) return rc == ROTGP_EINVAL ? fail(c, ROTGP_EUNSUPPORTED, "%s", c->err.c_str()) : rc;
+    ap.rt.set = true;
+    ap.rt.nseg = ap.nseg;
+    ap.rt.seg_chunks = ap.seg_chunks;
+    ap.rt.warm = ap.warm;
+    ap.rt.sh = ap.sh;
     // banded-inverse stencil: complex float, even N_x (TMA rows of 16-byte
     // multiples; the separate x-stencil kernel also wants N_x % 4 == 0)
     int K = 0, B = 0;
@@ -980,10 +992,28 @@ int tail_step(rotgp_ctx* c, int axis, bool imag, bool last) {
   return ROTGP_OK;
 }
 
+// May real time take the centred TMA sweeps on this axis?  Their weights m2 - 2,
+// al and be, of size up to 4 kappa, are rounded one by one, which moves the norm
+// by up to 1e-6 kappa^2 per step, the same way every step (measured 1.8e-9 at
+// kappa_z = 0.04, where the folded form moves it by 3e-10).  Up to 0.005 that is
+// 2.5e-11 per axis, within what the folded form itself does; 256 x 256 x 128 at
+// kappa 0.004 takes 87.5 us per step there, 128 folded.
+bool centred_ok(const rotgp_ctx* c, int axis) {
+  const double h = c->grid.h[axis];
+  return 0.25 * std::fabs(c->phys.dt) <= 0.005 * h * h;
+}
+
 int sweep(rotgp_ctx* c, int axis, bool imag, bool last) {
   if (tail_sweep(c, axis, imag)) return tail_step(c, axis, imag, last);
   const int mode = imag ? 1 : 0;
-  const AxisPlan& ap = c->axis[axis];
+  AxisPlan ap = c->axis[axis];
+  if (!imag && !c->fp64 && ap.sh.V == 1 && (ap.sh.C == 8 || ap.sh.C == 16) && ap.rt.set &&
+      (axis == 0 ? c->xmaps_ok && c->x_tma : c->smaps_ok) && !centred_ok(c, axis)) {
+    ap.nseg = ap.rt.nseg;
+    ap.seg_chunks = ap.rt.seg_chunks;
+    ap.warm = ap.rt.warm;
+    ap.sh = ap.rt.sh;
+  }
   stream_args a{};
   a.in = c->psi[c->cur];
   a.out = c->psi[1 - c->cur];

@@ -1,5 +1,5 @@
 """Real time in the one-line-per-lane TMA sweeps of complex float (the default
-of even rows in 3D) against the FP64 oracle: groups of lines and chunks partly
+of even rows in 3D up to kappa = 0.005) and beyond it against the FP64 oracle: groups of lines and chunks partly
 outside the grid, one and several segments per line, both chunk lengths, every
 ring depth.
 
@@ -23,10 +23,11 @@ CASES = [((32, 32, 32), None), ((34, 33, 31), None), ((130, 17, 70), None), ((18
          ((66, 40, 50), (16, 3, 2)), ((70, 34, 49), (16, 4, 1)), ((302, 130), (8, 5, 3))]
 
 
+@pytest.mark.parametrize("kappa", [0.0045, 0.02])
 @pytest.mark.parametrize("n,shape", CASES)
-def test_real_time_matches_oracle(n, shape):
+def test_real_time_matches_oracle(n, shape, kappa):
     h = tuple(10.0 / max(n) * f for f in (1.0, 1.02, 1.05))[:len(n)]
-    dt = 4.0 * 0.02 * h[0] ** 2
+    dt = 4.0 * kappa * h[0] ** 2
     grid = oracle.Grid(n, h)
     psi = oracle.init_analytic(grid, 1, inputs.random_phase_field(n[0], n[1], 3))
     psi = oracle.steps(grid, oracle.Phys(dt=min(dt, 2e-3), **KW), psi, 20, True)[0]
