@@ -29,8 +29,8 @@
 // system (A y = psi, psi' = 2y - psi: weights m2, al, be, no neighbour
 // points), TMA box loads and stores through R + 1 slots per warp, persistent
 // warps and programmatic launch; real time solves it in the centred form
-// (weight m2 - 2, see k_sweep_s1t), which holds the CN map's norm to rounding
-// as the folded form above does.
+// (weight m2 - 2, see k_sweep_s1t) where kappa is small, and the folded form
+// above elsewhere, each holding the CN map's norm to rounding.
 #pragma once
 
 #include "common.cuh"
