@@ -310,6 +310,7 @@ __global__ void __launch_bounds__(32) k_dcols(const dline_args a) {
 
 // ---------------------------------------------------------------- 2D steps
 constexpr int kDBits = 45, kDFrac = 40;
+constexpr int kDTries = 64;  // most repeats of an exchange (48 cross all scales)
 
 // v in units of 2^(ex - kDBits - kDFrac) as hi 2^kDFrac + lo; what is too
 // large, negative or NaN becomes the largest share
@@ -454,10 +455,20 @@ __global__ void __launch_bounds__(128) k_dsteps(const dstep_args a) {
           if (!meet(0, &z0, &z1)) s_fail = 1;
         }
         if (!s_fail && !meet(1, &hi, &lo)) s_fail = 1;
-        const int ex = s_ex, bits = 64 - __clzll(hi);
-        const int next = hi == 0 ? ex - 40 : hi >= most ? ex + 40 : ex + bits - kDBits - 1;
+        // The scale that this total asks for, from the bits of the whole total:
+        // a sum of many shares below one unit of hi lies in lo alone, and taken
+        // for nothing it would lower the scale until the shares are out of
+        // range again, and so on for ever.  With all bits a repeat leads to a
+        // total in range, or on in one direction to the end of the scales.
+        hi += lo >> kDFrac;
+        lo &= (1ull << kDFrac) - 1;
+        const int ex = s_ex, bits = hi ? kDFrac + 64 - __clzll(hi) : 64 - __clzll(lo);
+        const int next = hi >= most  ? ex + 40
+                         : bits == 0 ? ex - 40
+                                     : ex + bits - kDFrac - kDBits - 1;
         s_ex = max(-900, min(1000, next));
-        s_again = !s_fail && (hi < (1ull << (kDBits - 9)) || hi >= most) && s_ex != ex;
+        s_again = !s_fail && (hi < (1ull << (kDBits - 9)) || hi >= most) && s_ex != ex &&
+                  tries < kDTries;
         if (!s_again && !s_fail) {
           const double n = ldexp((double)hi + ldexp((double)lo, -kDFrac), ex - kDBits) * a.vol;
           const bool fine = hi > 0 && hi < most;

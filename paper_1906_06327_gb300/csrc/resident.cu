@@ -74,6 +74,7 @@ __device__ __forceinline__ float exp2i(int n) { return __uint_as_float((unsigned
 // Shares are integers in units of 2^(ex - kShareBits), a total of 2^ex being
 // 2^kShareBits; ex stays where the float factors exist.
 constexpr int kShareBits = 45, kExMin = -80, kExMax = 170;
+constexpr int kShareTries = 32;  // most repeats of an exchange (12 cross all scales)
 constexpr long long kShareMax = 1ll << (kShareBits + 2);
 // a compensated sum hi + lo (lo small) in those units, as hi 2^23 + lo in 32-bit
 // halves (64-bit conversions run in the double pipe); NaN and values out of
@@ -459,7 +460,7 @@ __global__ void __launch_bounds__(res_threads(H), 1) k_resident(const res_args a
       if (!y) __syncthreads();
     }
     // ---- the norm: this tile's share, then the total and the pending scale
-    for (;;) {
+    for (int tries = 0;; ++tries) {
       int2 v = share_of(acc.s, -acc.c, s_ex);
       v.x = __reduce_add_sync(0xffffffffu, v.x);
       v.y = __reduce_add_sync(0xffffffffu, v.y);
@@ -481,7 +482,8 @@ __global__ void __launch_bounds__(res_threads(H), 1) k_resident(const res_args a
         // the scale that this total asks for
         const int next = t == 0 ? ex - 40 : t >= kShareMax ? ex + 24 : ex + bits - kShareBits - 1;
         s_ex = max(kExMin, min(kExMax, next));
-        s_again = (t < (1ll << (kShareBits - 9)) || t >= kShareMax) && s_ex != ex;
+        s_again = (t < (1ll << (kShareBits - 9)) || t >= kShareMax) && s_ex != ex &&
+                  tries < kShareTries;
         const float h = (float)(int)(t >> 24) * 16777216.f, l = (float)(int)(t & 0xffffff);
         const float dn = exp2i(ex - kShareBits);
         const float2 sc = inv_sqrt(h * dn, l * dn, vol_h, vol_l);
