@@ -467,10 +467,11 @@ __global__ void __launch_bounds__(res_threads(H), 1) k_resident(const res_args a
       if (lane == 0) warp_part[warp] = v;
       __syncthreads();
       if (tid == 0) {
-        int hi = 0, lo = 0;
+        // (a warp's sums stay below 2^30, those of 512 threads pass 2^31)
+        long long hi = 0, lo = 0;
 #pragma unroll
         for (int i = 0; i < NW; ++i) hi += warp_part[i].x, lo += warp_part[i].y;
-        long long t = max(0ll, ((long long)hi << 23) + lo);
+        long long t = max(0ll, (hi << 23) + lo);
         unsigned long long* word = &a.sync->word[round & 1][0];
         post_share(word, min(t, kShareMax));
         t = poll_total(word, gridDim.x, &last[round & 1]);

@@ -3,8 +3,12 @@ from the one before them (random-phase starts lose most of their norm in the
 first step and little in the second), and totals that no scale of the shares
 holds at once.
 
+The on-chip stepper's tiles fill their CTAs from about 560 to 1,100 points a
+side: every thread then has a share, and the sums of a CTA are at their largest.
+
 Tolerances: complex double as tests/test_double_steps.py, 2e-15 per step against
-the chunked sweeps."""
+the chunked sweeps; complex float as tests/test_resident.py, 4 x 6e-8 per step
+and form, and the norm of a renormalised state within 1e-6."""
 import numpy as np
 import pytest
 
@@ -68,3 +72,70 @@ def test_zero_state_ends_in_an_error(precision):
     s.step_imag(3)
     with pytest.raises(RotgpError):
         s.sync()
+
+
+# one to three segments a thread, both short halos; 384 threads (halo above 8)
+FULL = [((560, 560), 0.006), ((600, 600), 0.006), ((600, 600), 0.02), ((800, 800), 0.006),
+        ((800, 800), 0.02), ((900, 900), 0.02), ((1024, 1024), 0.006), ((1100, 1100), 0.02),
+        ((1024, 768), 0.02), ((1000, 1000), 0.1)]
+
+
+def _flat(n):
+    """Density everywhere on the grid, a phase that varies slowly."""
+    x, y = np.meshgrid(np.linspace(0, 1, n[0] + 1), np.linspace(0, 1, n[1] + 1))
+    psi = np.exp(2j * np.pi * (x - 2 * y)) * (1 + 0.2 * np.sin(7 * x) * np.cos(5 * y))
+    psi[[0, -1]] = 0
+    psi[:, [0, -1]] = 0
+    return (psi / 12.0).astype(np.complex64)  # norm 1 on 12 x 12, to a few percent
+
+
+def _pair(n, kappa):
+    h = (12.0 / n[0], 12.0 / n[1])
+    s, t = (Solver(n, h, dt=4.0 * kappa * min(h) ** 2, **KW) for _ in range(2))
+    for ax in (0, 1):
+        t.set_solver(ax, "thomas")  # the sweep launches
+    return s, t
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,kappa", FULL)
+def test_full_tiles_norm(n, kappa):
+    s, t = _pair(n, kappa)
+    for x in (s, t):
+        x.set_psi(_flat(n), normalise=True)
+        x.step_imag(1)
+    assert abs(s.observables()["norm"] - 1) < 1e-6
+    for x in (s, t):
+        x.step_imag(19)
+        x.step_real(5)
+    assert abs(s.observables()["norm"] - 1) < 1e-6
+    ref = t.get_psi()
+    assert np.linalg.norm(s.get_psi() - ref) < 2 * 4 * 6e-8 * 25 * np.linalg.norm(ref)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [(800, 800), (1000, 1000)])
+def test_full_tiles_report_a_nan(n):
+    s, _ = _pair(n, 0.02)
+    psi = _flat(n)
+    psi[n[1] // 2, n[0] // 3] = np.nan
+    s.set_psi(psi)
+    s.step_imag(200)
+    with pytest.raises(RotgpError):
+        s.sync()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("scale", [1e3, 1e6])
+def test_full_tiles_normalise_a_large_state(scale):
+    """Shares of every thread beyond the first scale (a norm of 1e6 and 1e12)."""
+    n = (800, 800)
+    s, t = _pair(n, 0.02)
+    psi = _flat(n)
+    for x, f in ((s, scale), (t, 1.0)):
+        x.set_phys(g=0.0)
+        x.set_psi((psi * np.float32(f)).astype(np.complex64))
+        x.step_imag(4)
+    assert abs(s.observables()["norm"] - 1) < 1e-6
+    ref = t.get_psi()
+    assert np.linalg.norm(s.get_psi() - ref) < 2 * 4 * 6e-8 * 4 * np.linalg.norm(ref)
