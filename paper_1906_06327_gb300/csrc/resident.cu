@@ -81,7 +81,7 @@ constexpr long long kShareMax = 1ll << (kShareBits + 2);
 // range become the largest share (fminf drops the NaN)
 __device__ __forceinline__ int2 share_of(float hi, float lo, int ex) {
   const float up = exp2i(kShareBits - ex);
-  const float q = fminf(hi * up, (float)(kShareMax / 2));
+  const float q = fminf(hi * up, (float)kShareMax);
   const float top = floorf(q * (1.f / 8388608.f));
   const float rest = fmaf(top, -8388608.f, q) + fminf(fmaxf(lo * up, -8e6f), 8e6f);
   return make_int2((int)top, __float2int_rn(rest));

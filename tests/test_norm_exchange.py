@@ -139,3 +139,17 @@ def test_full_tiles_normalise_a_large_state(scale):
     assert abs(s.observables()["norm"] - 1) < 1e-6
     ref = t.get_psi()
     assert np.linalg.norm(s.get_psi() - ref) < 2 * 4 * 6e-8 * 4 * np.linalg.norm(ref)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("norm", [0.9, 1.9, 2.7, 3.8, 7.5])
+def test_first_norm_in_one_point(norm):
+    """A share as large as a total may be: the state in one point, the scale of
+    the shares just above 1 / (h_x h_y), Delta too short to spread it."""
+    n, h = (60, 44), (0.25, 0.2505)
+    psi = np.zeros((n[1] + 1, n[0] + 1), np.complex64)
+    psi[20, 30] = np.sqrt(norm / (h[0] * h[1]))
+    s = Solver(n, h, gamma=1.0, nu=1.0, g=0.0, omega=0.0, dt=1e-9)
+    s.set_psi(psi)
+    s.step_imag(1)
+    assert abs(s.observables()["norm"] - 1) < 1e-6
