@@ -325,11 +325,8 @@ __global__ void __launch_bounds__(res_threads(H), 1) k_resident(const res_args a
     auto h1 = [&](float2 p, int at, float x, float vy) {
       p = make_float2(pre * p.x, pre * p.y);
       if (IMAG) {
-        // s e^u psi = psi + ((s - 1) + s (e^u - 1)) psi: one rounding of psi
-        const float e =
-            exp_m1(-a.dt * fmaf(gs, fmaf(p.x, p.x, p.y * p.y), fmaf(a.hgam2 * x, x, vy)));
-        const float f = fmaf(sm1, e, e) + sm1;
-        A[at] = make_float2(fmaf(f, p.x, p.x), fmaf(f, p.y, p.y));
+        A[at] = damp(p, -a.dt * fmaf(gs, fmaf(p.x, p.x, p.y * p.y), fmaf(a.hgam2 * x, x, vy)),
+                     sm1);
       } else {
         // the advanced value rounded, and what the rounding left out (the x
         // sweep adds it to the change of its points)

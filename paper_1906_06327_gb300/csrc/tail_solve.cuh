@@ -24,16 +24,24 @@ __device__ __forceinline__ float2 change(const line_w& k, float2 psi, float2 f, 
       fmaf(k.g2.x, x, fmaf(-k.g2.y, y, fmaf(k.gc.x, psi.x, -(k.gc.y * psi.y)))),
       fmaf(k.g2.x, y, fmaf(k.g2.y, x, fmaf(k.gc.x, psi.y, k.gc.y * psi.x))));
 }
-// e^u - 1 to float accuracy relative to u: the Taylor series below 1/4, where
-// the steps of practice lie, and exp beyond.
-__device__ __forceinline__ float exp_m1(float u) {
-  float p = fmaf(u, 1.f / 5040.f, 1.f / 720.f);
-  p = fmaf(u, p, 1.f / 120.f);
-  p = fmaf(u, p, 1.f / 24.f);
-  p = fmaf(u, p, 1.f / 6.f);
-  p = fmaf(u, p, 0.5f);
-  p = fmaf(u * u, p, u);
-  return fabsf(u) < 0.25f ? p : __expf(u) - 1.f;
+// H1 of a point psi in imaginary time, (1 + m1) e^u psi.  Where u is small, as in
+// the steps of practice, psi + (m1 + (1 + m1) (e^u - 1)) psi with a Taylor series:
+// one rounding of psi.  From 1/4 on the product itself: formed as a change of
+// psi, a factor below 1e-7 came out as 0 and one of 1e-5 right to 1% (64 x 48 with u
+// down to -10: points off by up to 11%, now 2e-6).  Both factors are formed and
+// one taken: a branch made a 4096^2 step 3% slower.
+__device__ __forceinline__ float2 damp(float2 psi, float u, float m1) {
+  float q = fmaf(u, 1.f / 5040.f, 1.f / 720.f);
+  q = fmaf(u, q, 1.f / 120.f);
+  q = fmaf(u, q, 1.f / 24.f);
+  q = fmaf(u, q, 1.f / 6.f);
+  q = fmaf(u, q, 0.5f);
+  q = fmaf(u * u, q, u);
+  float e;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(u * 1.4426950408889634f));
+  const bool small = fabsf(u) < 0.25f;
+  const float f = small ? fmaf(m1, q, q) + m1 : fmaf(m1, e, e), b = small ? 1.f : 0.f;
+  return make_float2(fmaf(f, psi.x, b * psi.x), fmaf(f, psi.y, b * psi.y));
 }
 
 // cos(t) - 1 and sin(t) as rot_t (sweep_common.cuh) gives them: the Taylor

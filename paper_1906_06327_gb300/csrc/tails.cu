@@ -236,9 +236,7 @@ __global__ void __launch_bounds__(32 * kTailWarps, 2) k_tail_x(const tail_args a
       const float pot = fmaf(a.hgam2 * x, x, vy);
       if (IMAG) {
         const float gg = near ? gs : a.g;
-        const float q = exp_m1(-a.dt * fmaf(gg, fmaf(p.x, p.x, p.y * p.y), pot));
-        const float f = fmaf(m1, q, q) + m1;
-        row[e] = make_float2(fmaf(f, p.x, p.x), fmaf(f, p.y, p.y));
+        row[e] = damp(p, -a.dt * fmaf(gg, fmaf(p.x, p.x, p.y * p.y), pot), m1);
       } else {
         const float2 v = make_float2(fmaf(m1, p.x, p.x), fmaf(m1, p.y, p.y));
         float2 w, rest;
