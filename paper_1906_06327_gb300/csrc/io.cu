@@ -110,9 +110,11 @@ __global__ void __launch_bounds__(256) k_load(const cpx<TS>* __restrict__ src,
   }
 }
 
-// s v rounded once
+// s v rounded once, s = sh + sl; infinities, of which the second part makes NaN,
+// take the product in double
 __device__ __forceinline__ float scaled(double s, float sh, float sl, float v, float) {
-  return fmaf(sh, v, sl * v);
+  const float r = fmaf(sh, v, sl * v);
+  return isfinite(r) ? r : (float)(s * (double)v);
 }
 template <class TS, class TD>
 __device__ __forceinline__ TD scaled(double s, float, float, TS v, TD) {
