@@ -1937,6 +1937,7 @@ int rotgp_tune(rotgp_ctx* c, int axis, int lines_per_lane, int chunk, int ring,
     ap.hcs = segments;
     ap.hpc = pc;
     ap.hlsub = ls;
+    c->user_plan = true;
     return ROTGP_OK;
   }
   if (warps_per_block < 1 || warps_per_block > 8)

@@ -1,0 +1,32 @@
+"""Forms and shapes that were asked for are the ones that run: contexts whose
+default plan takes kernels of its own (tiles with long halos, the on-chip stepper)
+against contexts with the same forms asked for from the start, bit for bit."""
+import numpy as np
+import pytest
+
+from paper_1906_06327_gb300.rotgp import Solver
+
+pytestmark = pytest.mark.gpu
+
+KW = dict(gamma=1.0, nu=1.1, g=20.0, omega=0.4)
+
+
+def _run(s, imag=True):
+    s.init_analytic(1, seed=4)
+    s.step_imag(3) if imag else s.step_real(3)
+    return s.get_psi()
+
+
+@pytest.mark.parametrize("imag", [True, False])
+def test_tuned_exact_solve_runs(imag):
+    """A halo of 32 points: the exact solve is the form that rotgp_tune shapes,
+    the default runs tiles."""
+    n, h = (300, 300), (0.1, 0.1)
+    a, b = (Solver(n, h, dt=4 * 1.15 * 0.01, **KW) for _ in range(2))
+    for ax in (0, 1):
+        b.set_solver(ax, "hybrid")
+    for s in (a, b):
+        for ax in (0, 1):
+            s.tune(ax, 1, 8, 3, 1, 2)
+        assert s.info()["hybrid_cluster"] == [2, 2]
+    assert np.array_equal(_run(a, imag), _run(b, imag))
