@@ -2039,7 +2039,17 @@ int rotgp_autotune(rotgp_ctx* c, int steps, int* choice) {
   const size_t state = (size_t)c->sites * c->elem;
   const int cur0 = c->cur;
   const long long steps0 = c->steps;
-  const bool prof0 = c->prof, plan0 = c->user_plan;
+  const bool prof0 = c->prof, plan0 = c->user_plan, fuse0 = c->fuse_xy;
+  const std::array<AxisPlan, 3> axes0{c->axis[0], c->axis[1], c->axis[2]};
+  // the forms and shapes as they were (the stencil weights stay as built since)
+  auto plan_before = [&] {
+    for (int a = 0; a < dim; ++a) {
+      const bool fresh = c->axis[a].wtab_fresh;
+      c->axis[a] = axes0[a];
+      c->axis[a].wtab_fresh = fresh;
+    }
+    c->fuse_xy = fuse0;
+  };
   c->prof = false;
   c->user_plan = true;  // the sweep forms first
   double* saved_scale = reinterpret_cast<double*>(static_cast<char*>(c->staging) + state);
@@ -2154,18 +2164,27 @@ int rotgp_autotune(rotgp_ctx* c, int steps, int* choice) {
     }
     ap.lsegs = best_s;
   }
-  // and the default plan where it has kernels that take no form or shape
+  // and the default plan where it has kernels that take no form or shape, with
+  // the forms of the axes that those do not serve as they were
   if (e == cudaSuccess && !rc) {
+    const std::array<AxisPlan, 3> tuned{c->axis[0], c->axis[1], c->axis[2]};
+    const bool fused = c->fuse_xy;
+    plan_before();
     c->user_plan = false;
     float ms = 0;
-    if ((resident(c, true) || double_steps(c, true) || tail_sweep(c, 0, true)) &&
-        time_current(&ms) && ms < best_ms)
+    const bool own = resident(c, true) || double_steps(c, true) || tail_sweep(c, 0, true);
+    if (own && time_current(&ms) && ms < best_ms) {
       best = 0;
-    else
+    } else {
+      for (int a = 0; a < dim; ++a) c->axis[a] = tuned[a];
+      c->fuse_xy = fused;
       c->user_plan = true;
-    if (!c->user_plan && e == cudaSuccess && !rc) rc = apply(0);
+    }
   }
-  if (e != cudaSuccess || rc) c->user_plan = plan0;
+  if (e != cudaSuccess || rc) {
+    plan_before();
+    c->user_plan = plan0;
+  }
   for (cudaEvent_t x : ev)
     if (x) cudaEventDestroy(x);
   const cudaError_t er = restore();
