@@ -942,10 +942,17 @@ int xy_pass(rotgp_ctx* c, bool imag) {
 // sweeps cannot read (255 x 256 x 128 167 us against 194 in imaginary time, 171
 // against 233 in real time; 65 x 49 x 33 27 against 36).  On even rows the TMA
 // sweeps are the faster ones (256 x 256 x 128 67 us in imaginary and 87 us in
-// real time, against 145 in tiles).
+// real time, against 145 in tiles).  Short lines with a halo above 16 stay in the
+// exact partition solve as long as one wave of its tiles takes them all: a tile
+// of tails runs H + L points in sequence whatever the length, a thread of the
+// exact solve only a sixteenth of the line (2D 32^2, halo 21: 33 us in tails, 19 in
+// the exact solve; 64^2, halo 56: 31 / 21; 128^2, halo 33: 23 / 23, halo 59: 29 / 23;
+// 256^2, halo 35: 25 / 31; 48^3: 42 / 25; 64^3: 39 / 31; 96^3: 35 / 58).
 bool tail_sweep(const rotgp_ctx* c, int axis, bool imag) {
-  return !c->fp64 && !c->user_plan && c->tails[axis][imag ? 1 : 0].blocks > 0 &&
-         (c->halo > 16 || c->nx % 2 != 0);
+  const AxisPlan& ap = c->axis[axis];
+  if (c->fp64 || c->user_plan || c->tails[axis][imag ? 1 : 0].blocks == 0) return false;
+  if (c->halo <= 16) return c->nx % 2 != 0;
+  return !ap.use_hybrid || ap.len >= 2 * c->halo + 32 || ap.lines >= 8192;
 }
 
 int tail_step(rotgp_ctx* c, int axis, bool imag, bool last) {

@@ -45,3 +45,15 @@ def test_autotune_that_keeps_the_default_plan(n, kappa):
     assert choice == 0 and a.info() == b.info()
     assert np.array_equal(_run(a), _run(b))
     assert np.array_equal(_run(a, False), _run(b, False))
+
+
+@pytest.mark.parametrize("n,kappa", [((32, 32), 0.5), ((64, 64), 1.15), ((63, 65), 1.15),
+                                     ((48, 48, 48), 1.15)])
+def test_short_lines_with_long_halos_take_the_exact_solve(n, kappa):
+    """Where tiles of tails would be the slower ones."""
+    kw = dict(KW, lam=1.0, dt=4 * kappa * 0.01)
+    a, b = (Solver(n, (0.1,) * len(n), **kw) for _ in range(2))
+    for ax in range(len(n)):
+        b.set_solver(ax, "hybrid")
+    assert np.array_equal(_run(a), _run(b))
+    assert np.array_equal(_run(a, False), _run(b, False))
