@@ -378,8 +378,14 @@ int rotgp_observables_noalloc(const rotgp_grid* grid, const rotgp_phys* phys, in
  *    axes and one CTA per line (rotgp_tune segments = 1).
  *  ROTGP_BATCH_GRAPH  the instances' own kernels, captured once as a CUDA
  *    graph (fork from the batch stream into the instance streams, join
- *    back) and replayed; results equal those of single contexts bit for bit.
- *  ROTGP_BATCH_DIRECT  the same kernels launched directly.
+ *    back) and replayed; results equal those of single contexts bit for bit,
+ *    except where several 2D instances in their default plan would each run
+ *    blocks of steps over the whole chip (see rotgp_set_solver), one after
+ *    another, and are done sooner side by side in sweeps: results then equal
+ *    up to rounding and the truncation bound (for complex float and even N_x
+ *    bit for bit those of single contexts with ROTGP_SOLVER_THOMAS).
+ *  ROTGP_BATCH_DIRECT  the instances' own kernels launched directly; results
+ *    equal those of single contexts bit for bit.
  * All calls are ordered after earlier work on the caller's stream and
  * before its later work. */
 #define ROTGP_BATCH_DIRECT 0

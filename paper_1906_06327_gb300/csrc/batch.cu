@@ -16,6 +16,7 @@
 // mu is compared with its value one check earlier; an instance is converged
 // when the relative change is below the tolerance and its vortex count did
 // not change, and later graphs leave it out.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -95,6 +96,28 @@ int observe_set(rotgp_batch* b, const std::vector<int>& set, rotgp_obs* out) {
   return first;
 }
 
+// Would the instances of `set` that can step in launches over the whole chip, one
+// after another, be done sooner by their sweeps, side by side?  Many small ones
+// would: a launch over the chip takes 3 to 5 us per step however small the state,
+// while a graph keeps many sweeps in flight, none of which fills the chip (per
+// step of 64 instances of 128^2 201 us one after another, 49 side by side; 16 of
+// 256^2 53 / 23, 16 of 512^2 73 / 77, 4 of 128^2 13 / 12, 2 of 128^2 6.5 / 12; complex
+// double, 32 of 128^2 400 / 115).  Launched one by one (DIRECT) the sweeps are the
+// slower ones in every case (64 of 128^2 212 / 284 us).
+bool side_by_side(rotgp_batch* b, const std::vector<int>& set, long long n, bool imag) {
+  double alone = 0, beside = 0, least = 0;
+  int count = 0;
+  for (int i : set) {
+    if (!rotgp::ctx_resident(b->ctx[i], imag)) continue;
+    const rotgp::ctx_cost t = rotgp::ctx_step_cost(b->ctx[i], imag, n);
+    alone += t.alone;
+    beside += t.beside;
+    least = std::max(least, t.least);
+    ++count;
+  }
+  return count > 1 && least + beside < alone;
+}
+
 // Run n steps of the instances in `set` (mode: ROTGP_BATCH_*), ordered after
 // the caller's stream and before its next work.
 int run_set(rotgp_batch* b, const std::vector<int>& set, long long n, bool imag, int mode) {
@@ -102,7 +125,10 @@ int run_set(rotgp_batch* b, const std::vector<int>& set, long long n, bool imag,
   cudaError_t e = cudaEventRecord(b->user_ev, b->user);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->user_ev, 0);
   if (e != cudaSuccess) return bfail(b, ROTGP_ECUDA, "order: %s", cudaGetErrorString(e));
+  const bool beside = mode == ROTGP_BATCH_GRAPH && side_by_side(b, set, n, imag);
+  for (int i : set) rotgp::ctx_set_beside(b->ctx[i], beside);
   const int rc = run_set_inner(b, set, n, imag, mode);
+  for (int i : set) rotgp::ctx_set_beside(b->ctx[i], false);
   e = cudaEventRecord(b->user_ev, b->stream);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(b->user, b->user_ev, 0);
   if (!rc && e != cudaSuccess) return bfail(b, ROTGP_ECUDA, "order: %s", cudaGetErrorString(e));

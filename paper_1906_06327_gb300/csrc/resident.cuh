@@ -71,6 +71,15 @@ cudaError_t launch_res_tables(float2* tab, int nlines, int iters, const axis_coe
 
 // Does a step of this mode of the context run in the on-chip stepper?
 bool ctx_resident(const rotgp_ctx* c, bool imag);
+// Its time per step of a block of n: alone, one launch over the whole chip; or
+// in launches of its own beside other instances', what it adds to them, and the
+// least time of a step.
+struct ctx_cost {
+  double alone, beside, least;
+};
+ctx_cost ctx_step_cost(const rotgp_ctx* c, bool imag, long long n);
+// Steps from here on beside other instances' (no launch over the whole chip).
+void ctx_set_beside(rotgp_ctx* c, bool on);
 // Points over which a line carry of the context stays above the rounding of
 // the exact partition solve (hybrid.cuh).
 int ctx_carry_reach(const rotgp_ctx* c);

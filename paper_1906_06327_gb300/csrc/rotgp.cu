@@ -122,6 +122,7 @@ struct rotgp_ctx {
   // on-chip 2D stepper (resident.cu): complex float, while the plan is the
   // default one (no form or shape asked for); plans and tables per mode
   bool user_plan = false;
+  bool beside = false;  // one of several that step side by side: no launch over the whole chip
   bool res_ok[2] = {false, false};
   res_plan rplan[2];
   // weights of the two-tail line solve [axis][mode], and the tiles of its
@@ -745,7 +746,7 @@ bool double_steps(const rotgp_ctx* c, bool imag) {
   return imag && c->fp64 && c->d_rows && !c->user_plan && c->chunk_ok;
 }
 bool double_blocks(const rotgp_ctx* c, bool imag) {
-  return double_steps(c, imag) && c->d_sync && dstep_fits(c->nx, c->ny, c->halo);
+  return double_steps(c, imag) && c->d_sync && !c->beside && dstep_fits(c->nx, c->ny, c->halo);
 }
 
 int double_block(rotgp_ctx* c, long long n) {
@@ -833,7 +834,7 @@ int double_sweep(rotgp_ctx* c, int axis, bool last) {
 // states whose tiles fit the shared memory and whose carries need a halo of
 // at most 16 points, unless a form or shape was asked for.
 bool resident(const rotgp_ctx* c, bool imag) {
-  return c->res_ok[imag ? 1 : 0] && !c->user_plan && c->chunk_ok &&
+  return c->res_ok[imag ? 1 : 0] && !c->user_plan && !c->beside && c->chunk_ok &&
          c->halo <= c->rplan[imag ? 1 : 0].H + 2;
 }
 
@@ -1298,6 +1299,32 @@ int ctx_carry_reach(const rotgp_ctx* c) {
 }
 bool ctx_resident(const rotgp_ctx* c, bool imag) {
   return resident(c, imag) || double_blocks(c, imag);
+}
+void ctx_set_beside(rotgp_ctx* c, bool on) { c->beside = on; }
+ctx_cost ctx_step_cost(const rotgp_ctx* c, bool imag, long long n) {
+  // Microseconds on GB300: straight lines through graphs of 2 to 64 instances of
+  // 64^2 to 900^2 points (complex double to 300^2) in blocks of 20 or 50 steps and
+  // calls of 1 to 3 steps, each decision among them right to 5% of the faster
+  // way, but for 8 x 512^2 with a halo of 10 and 2 x 300^2 in double (15%).
+  const double s = (double)c->sites, per = 1.0 / (double)std::max(1LL, n);
+  if (c->fp64) {
+    // lines of 128 P points, a CTA's rounds of both sweeps
+    const int longest = std::max(c->nx, c->ny);
+    const double rounds = (c->nx + c->sm_count - 1) / c->sm_count + (c->ny + c->sm_count - 1) / c->sm_count;
+    const int P = longest <= 128 ? 1 : longest <= 256 ? 2 : longest <= 512 ? 4 : 8;
+    return {16.0 * per + rounds * (5.0 + 0.9 * P), 0.2 + 2.2e-4 * s, 33.0};
+  }
+  const bool near = c->halo <= 8;
+  const double alone = (9.3 + 5e-6 * s) * per + (near ? 3.0 + 6e-6 * s : 4.5 + 1.35e-5 * s);
+  // the sweeps of run_steps: tiles, one-line TMA forms, or the folded forms
+  if (c->nx % 2 != 0) return {alone, 0.3 + 5e-6 * s, 15.5};
+  bool one_line = true;
+  for (int a = 0; a < 2; ++a)
+    one_line = one_line && c->axis[a].sh.V == 1 && (imag || centred_ok(c, a));
+  if (one_line && imag) return {alone, 0.3 + 1.3e-5 * s, 11.0};
+  if (one_line) return {alone, 0.35 + 2.4e-5 * s, 12.2};
+  if (imag) return {alone, 0.35 + 1.4e-5 * s, 27.0};
+  return near ? ctx_cost{alone, 0.4 + 1.9e-5 * s, 25.0} : ctx_cost{alone, 0.5 + 5e-5 * s, 44.0};
 }
 long long ctx_plan_version(const rotgp_ctx* c) { return c->plan_version; }
 void ctx_add_steps(rotgp_ctx* c, long long n) { c->steps += n; }
