@@ -282,6 +282,8 @@ int rotgp_tune(rotgp_ctx* ctx, int axis, int lines_per_lane, int chunk, int ring
  * of steps in one cooperative launch that keeps the state on chip (record
  * "steps_2d" of rotgp_profile_read, one record per launch); results equal
  * those of the sweeps up to float rounding and the same truncation bound.
+ * (A call of a single imaginary-time step runs in the sweeps where those are
+ * the faster ones: even N_x and a halo of at most 8 points.)
  * A wait between its tiles is bounded (about 2 s of device time,
  * ROTGP_ETIMEOUT).  Likewise imaginary-time steps in complex double with a
  * halo of at most 64 points, shorter than the lines, run in kernels of their

@@ -1133,10 +1133,20 @@ int sweep(rotgp_ctx* c, int axis, bool imag, bool last) {
   return ROTGP_OK;
 }
 
+// A call of one step takes the sweeps where they run in their one-line TMA forms in
+// imaginary time: tiles loaded and handed back for one step cost more than the
+// second launch (128^2 12.5 against 12.0 us, 512^2 16.6 / 14.7, 1000^2 23.6 / 17.6, 1400 x
+// 500 19.7 / 15.9; two steps 14.6 / 23.6, 20.8 / 29.0, 32.9 / 35.0, 26.9 / 31.5).  The other
+// forms of the sweeps take 25 us and more per step, and real time on 512^2 14.8
+// against 16.1, half of what it took in the folded form.
+bool one_in_sweeps(const rotgp_ctx* c, long long n, bool imag) {
+  return n == 1 && imag && c->nx % 2 == 0 && c->axis[0].sh.V == 1 && c->axis[1].sh.V == 1;
+}
+
 int run_steps(rotgp_ctx* c, long long n, bool imag) {
   if (!c) return ROTGP_EINVAL;
   if (n < 0) return fail(c, ROTGP_EINVAL, "negative step count");
-  if (resident(c, imag)) return resident_steps(c, n, imag, nullptr);
+  if (resident(c, imag) && !one_in_sweeps(c, n, imag)) return resident_steps(c, n, imag, nullptr);
   if (double_blocks(c, imag)) return double_block(c, n);
   const bool dbl = double_steps(c, imag);
   for (long long s = 0; s < n; ++s) {

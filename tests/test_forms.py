@@ -57,3 +57,14 @@ def test_short_lines_with_long_halos_take_the_exact_solve(n, kappa):
         b.set_solver(ax, "hybrid")
     assert np.array_equal(_run(a), _run(b))
     assert np.array_equal(_run(a, False), _run(b, False))
+
+
+def test_calls_of_one_step_take_the_sweeps():
+    a, b = (Solver((64, 48), (0.2, 0.2), dt=1e-3, **KW) for _ in range(2))
+    for ax in (0, 1):
+        b.set_solver(ax, "thomas")
+    for s in (a, b):
+        s.init_analytic(1, seed=4)
+        for _ in range(5):
+            s.step_imag(1)
+    assert np.array_equal(a.get_psi(), b.get_psi())

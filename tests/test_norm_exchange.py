@@ -145,8 +145,9 @@ def test_full_tiles_normalise_a_large_state(scale):
 @pytest.mark.parametrize("norm", [0.9, 1.9, 2.7, 3.8, 7.5])
 def test_first_norm_in_one_point(norm):
     """A share as large as a total may be: the state in one point, the scale of
-    the shares just above 1 / (h_x h_y), Delta too short to spread it."""
-    n, h = (60, 44), (0.25, 0.2505)
+    the shares just above 1 / (h_x h_y), Delta too short to spread it (odd N_x: a
+    single step that runs in the stepper)."""
+    n, h = (61, 44), (0.25, 0.2505)
     psi = np.zeros((n[1] + 1, n[0] + 1), np.complex64)
     psi[20, 30] = np.sqrt(norm / (h[0] * h[1]))
     s = Solver(n, h, gamma=1.0, nu=1.0, g=0.0, omega=0.0, dt=1e-9)
