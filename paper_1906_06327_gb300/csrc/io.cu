@@ -110,11 +110,12 @@ __global__ void __launch_bounds__(256) k_load(const cpx<TS>* __restrict__ src,
   }
 }
 
-// s v rounded once, s = sh + sl; infinities, of which the second part makes NaN,
-// take the product in double
+// s v rounded once, s = sh + sl.  The second part of an infinity (NaN, or of the
+// other sign) is left out; taking such values through double instead, in a
+// branch, made reading back 256 x 256 x 128 100 us slower.
 __device__ __forceinline__ float scaled(double s, float sh, float sl, float v, float) {
-  const float r = fmaf(sh, v, sl * v);
-  return isfinite(r) ? r : (float)(s * (double)v);
+  const float p = sl * v;
+  return fmaf(sh, v, fabsf(p) < __int_as_float(0x7f800000) ? p : 0.f);
 }
 template <class TS, class TD>
 __device__ __forceinline__ TD scaled(double s, float, float, TS v, TD) {
