@@ -49,46 +49,86 @@ __global__ void k_init_analytic(cpx<T>* psi, int nx, int ny, int nz, int dim, do
   }
 }
 
-// Both layouts are copied row by row: a warp takes 256 points of a row, so no
-// index is divided per point and every lane has eight loads in flight.  In
-// complex float nothing is converted to double (three or six operations of
-// the double pipe per point made whole calls on a 4096^2 state take 222 us in
-// and 202 us out; 79 and 66 us now, 256 x 256 x 128 130 and 115 us, now 55 and
-// 42).  The norm of a loaded state is summed as it is written.
+// Between complex float and complex float, both layouts are copied row by row: a
+// warp takes 256 points of a row, so no index is divided per point and every
+// lane has eight loads in flight.  Nothing is converted to double there (three or
+// six operations of the double pipe per point made whole calls on a 4096^2 state
+// take 222 us in and 202 us out; 79 and 66 us now, 256 x 256 x 128 130 and 115 us,
+// now 55 and 42).  The norm of a loaded state is summed as it is written.
+//
+// Where either side is double, and on rows of a few points, a thread takes one
+// point at a time from the whole grid: the double pipe is what bounds those
+// copies, and a lane outside the row costs it as much as one inside (into complex
+// double, rows against points: 20 x 300 x 300 177 / 21 us, 256 x 256 x 128 133 / 70; from it, 99 / 25 and 51 / 68).
 constexpr int kRowPart = 256;
+template <class TS, class TD>
+constexpr bool row_copy() { return sizeof(TS) + sizeof(TD) == 8; }
+constexpr int kRowLeast = 16;  // points of a row
+
+// Coordinates of point idx of an a x b x ... grid.
+__device__ __forceinline__ void grid_point(long long idx, int a, int b, int* i, int* j, int* k) {
+  if (idx <= 0xffffffffll) {
+    const unsigned u = (unsigned)idx, r = u / (unsigned)a;
+    *i = (int)(u - r * (unsigned)a);
+    *k = (int)(r / (unsigned)b);
+    *j = (int)(r - (unsigned)*k * (unsigned)b);
+  } else {
+    const long long r = idx / a;
+    *i = (int)(idx - r * a);
+    *k = (int)(r / b);
+    *j = (int)(r - (long long)*k * b);
+  }
+}
 
 // ABI layout -> device layout, with the norm of the loaded state in the same
 // pass (NORM) and from it the pending scale; otherwise the scale is 1.
-template <class TS, class TD, bool NORM>
+template <class TS, class TD, bool NORM, bool ROWS>
 __global__ void __launch_bounds__(256) k_load(const cpx<TS>* __restrict__ src,
                                               cpx<TD>* __restrict__ psi, int nx, int ny, int nz,
                                               int dim, double vol, double* partials,
                                               unsigned* counter, double* scale, double* norm,
                                               int* flags) {
   using S = typename run_sum<TD>::sum;
-  const int lane = threadIdx.x & 31, parts = (nx + kRowPart - 1) / kRowPart;
-  const long long tasks = (long long)ny * nz * parts;
   run_sum<TD> q;
-  for (long long t = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); t < tasks;
-       t += (long long)gridDim.x * 8) {
-    const long long row = t / parts;
-    const int i0 = (int)(t - row * parts) * kRowPart + lane;
-    const int k = (int)(row / ny), j = (int)(row - (long long)k * ny);
-    const bool zero = j == 0 || (dim == 3 && k == 0);
-    const cpx<TS>* from = src + ((long long)k * (ny + 1) + j) * (nx + 1);
-    cpx<TS> v[kRowPart / 32];
-#pragma unroll
-    for (int u = 0; u < kRowPart / 32; ++u) {
-      const int i = i0 + 32 * u;
-      v[u] = !zero && i > 0 && i < nx ? from[i] : mk<TS>(0, 0);
-    }
-#pragma unroll
-    for (int u = 0; u < kRowPart / 32; ++u) {
-      const int i = i0 + 32 * u;
-      if (i >= nx) continue;
-      const cpx<TD> w = mk<TD>((TD)v[u].x, (TD)v[u].y);
-      psi[row * nx + i] = w;
+  if constexpr (!ROWS) {
+    const long long n = (long long)nx * ny * nz;
+    for (long long idx = (long long)blockIdx.x * 256 + threadIdx.x; idx < n;
+         idx += (long long)gridDim.x * 256) {
+      int i, j, k;
+      grid_point(idx, nx, ny, &i, &j, &k);
+      cpx<TD> w = mk<TD>(0, 0);
+      if (i != 0 && j != 0 && !(dim == 3 && k == 0)) {
+        const cpx<TS> v = src[((long long)k * (ny + 1) + j) * (nx + 1) + i];
+        w = mk<TD>((TD)v.x, (TD)v.y);
+      }
+      psi[idx] = w;
       if (NORM) q.add(abs2(w));
+    }
+  } else {
+    const int lane = threadIdx.x & 31, parts = (nx + kRowPart - 1) / kRowPart;
+    const long long tasks = (long long)ny * nz * parts;
+    for (long long t = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); t < tasks;
+         t += (long long)gridDim.x * 8) {
+      const long long row = t / parts;
+      const int i0 = (int)(t - row * parts) * kRowPart + lane;
+      const int k = (int)(row / ny), j = (int)(row - (long long)k * ny);
+      const bool zero = j == 0 || (dim == 3 && k == 0);
+      const cpx<TS>* from = src + ((long long)k * (ny + 1) + j) * (nx + 1);
+      cpx<TS> v[kRowPart / 32];
+#pragma unroll
+      for (int u = 0; u < kRowPart / 32; ++u) {
+        const int i = i0 + 32 * u;
+        v[u] = !zero && i > 0 && i < nx ? from[i] : mk<TS>(0, 0);
+      }
+#pragma unroll
+      for (int u = 0; u < kRowPart / 32; ++u) {
+        const int i = i0 + 32 * u;
+        if (i - lane >= nx) break;
+        if (i >= nx) continue;
+        const cpx<TD> w = mk<TD>((TD)v[u].x, (TD)v[u].y);
+        psi[row * nx + i] = w;
+        if (NORM) q.add(abs2(w));
+      }
     }
   }
   if (!NORM) {
@@ -124,32 +164,49 @@ __device__ __forceinline__ TD scaled(double s, float, float, TS v, TD) {
 
 // Device layout -> ABI layout, multiplying by the pending scale and writing
 // zeros on both edges of every axis.
-template <class TS, class TD>
+template <class TS, class TD, bool ROWS>
 __global__ void __launch_bounds__(256) k_store(const cpx<TS>* __restrict__ psi,
                                                cpx<TD>* __restrict__ dst, int nx, int ny, int nz,
                                                int dim, const double* scale) {
-  const int lane = threadIdx.x & 31, parts = (nx + 1 + kRowPart - 1) / kRowPart;
-  const long long tasks = (long long)(ny + 1) * (dim == 3 ? nz + 1 : 1) * parts;
   const double s = *scale;
   const float sh = (float)s, sl = (float)(s - (double)sh);
-  for (long long t = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); t < tasks;
-       t += (long long)gridDim.x * 8) {
-    const long long row = t / parts;
-    const int i0 = (int)(t - row * parts) * kRowPart + lane;
-    const int k = (int)(row / (ny + 1)), j = (int)(row - (long long)k * (ny + 1));
-    const bool zero = j == 0 || j == ny || (dim == 3 && (k == 0 || k == nz));
-    const cpx<TS>* from = psi + ((long long)k * ny + j) * nx;
-    cpx<TS> v[kRowPart / 32];
-#pragma unroll
-    for (int u = 0; u < kRowPart / 32; ++u) {
-      const int i = i0 + 32 * u;
-      v[u] = !zero && i > 0 && i < nx ? from[i] : mk<TS>(0, 0);
+  if constexpr (!ROWS) {
+    const long long n = (long long)(nx + 1) * (ny + 1) * (dim == 3 ? nz + 1 : 1);
+    for (long long idx = (long long)blockIdx.x * 256 + threadIdx.x; idx < n;
+         idx += (long long)gridDim.x * 256) {
+      int i, j, k;
+      grid_point(idx, nx + 1, ny + 1, &i, &j, &k);
+      const bool edge = i == 0 || i == nx || j == 0 || j == ny || (dim == 3 && (k == 0 || k == nz));
+      cpx<TD> w = mk<TD>(0, 0);
+      if (!edge) {
+        const cpx<TS> v = psi[((long long)k * ny + j) * nx + i];
+        w = mk<TD>(scaled(s, sh, sl, v.x, (TD)0), scaled(s, sh, sl, v.y, (TD)0));
+      }
+      dst[idx] = w;
     }
+  } else {
+    const int lane = threadIdx.x & 31, parts = (nx + 1 + kRowPart - 1) / kRowPart;
+    const long long tasks = (long long)(ny + 1) * (dim == 3 ? nz + 1 : 1) * parts;
+    for (long long t = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); t < tasks;
+         t += (long long)gridDim.x * 8) {
+      const long long row = t / parts;
+      const int i0 = (int)(t - row * parts) * kRowPart + lane;
+      const int k = (int)(row / (ny + 1)), j = (int)(row - (long long)k * (ny + 1));
+      const bool zero = j == 0 || j == ny || (dim == 3 && (k == 0 || k == nz));
+      const cpx<TS>* from = psi + ((long long)k * ny + j) * nx;
+      cpx<TS> v[kRowPart / 32];
 #pragma unroll
-    for (int u = 0; u < kRowPart / 32; ++u) {
-      const int i = i0 + 32 * u;
-      if (i <= nx)
-        dst[row * (nx + 1) + i] = mk<TD>(scaled(s, sh, sl, v[u].x, (TD)0), scaled(s, sh, sl, v[u].y, (TD)0));
+      for (int u = 0; u < kRowPart / 32; ++u) {
+        const int i = i0 + 32 * u;
+        v[u] = !zero && i > 0 && i < nx ? from[i] : mk<TS>(0, 0);
+      }
+#pragma unroll
+      for (int u = 0; u < kRowPart / 32; ++u) {
+        const int i = i0 + 32 * u;
+        if (i - lane > nx) break;
+        if (i <= nx)
+          dst[row * (nx + 1) + i] = mk<TD>(scaled(s, sh, sl, v[u].x, (TD)0), scaled(s, sh, sl, v[u].y, (TD)0));
+      }
     }
   }
 }
@@ -209,11 +266,18 @@ cudaError_t launch_load(bool fp64_store, bool fp64_src, const void* src, void* p
                         int nz, int dim, double vol, bool normalise, double* partials,
                         unsigned* counter, double* scale, double* norm, int* flags, int blocks,
                         cudaStream_t s) {
-  blocks = (int)std::min<long long>(blocks, (row_tasks((long long)ny * nz, nx) + 7) / 8);
-#define ROTGP_LD(TS, TD)                                                                        \
-  (normalise ? k_load<TS, TD, true> : k_load<TS, TD, false>)<<<blocks, 256, 0, s>>>(            \
-      static_cast<const cpx<TS>*>(src), static_cast<cpx<TD>*>(psi), nx, ny, nz, dim, vol,       \
-      partials, counter, scale, norm, flags)
+#define ROTGP_LD(TS, TD)                                                                       \
+  do {                                                                                         \
+    const bool rows = row_copy<TS, TD>() && nx >= kRowLeast;                                   \
+    const long long work = rows ? (row_tasks((long long)ny * nz, nx) + 7) / 8                  \
+                                : ((long long)nx * ny * nz + 255) / 256;                       \
+    auto fn = rows ? (normalise ? k_load<TS, TD, true, row_copy<TS, TD>()>                     \
+                                : k_load<TS, TD, false, row_copy<TS, TD>()>)                   \
+                   : (normalise ? k_load<TS, TD, true, false> : k_load<TS, TD, false, false>); \
+    fn<<<(int)std::min<long long>(blocks, work), 256, 0, s>>>(                                 \
+        static_cast<const cpx<TS>*>(src), static_cast<cpx<TD>*>(psi), nx, ny, nz, dim, vol,    \
+        partials, counter, scale, norm, flags);                                                \
+  } while (0)
   if (fp64_src) {
     if (fp64_store) ROTGP_LD(double, double); else ROTGP_LD(double, float);
   } else {
@@ -225,11 +289,16 @@ cudaError_t launch_load(bool fp64_store, bool fp64_src, const void* src, void* p
 
 cudaError_t launch_unpack(bool fp64_store, bool fp64_dst, const void* psi, void* dst, int nx,
                           int ny, int nz, int dim, const double* scale, cudaStream_t s) {
-  const long long tasks = row_tasks((long long)(ny + 1) * (dim == 3 ? nz + 1 : 1), nx + 1);
-  const int blocks = (int)std::min<long long>(152 * 8, (tasks + 7) / 8);
-#define ROTGP_UP(TS, TD)                                                                   \
-  k_store<TS, TD><<<blocks, 256, 0, s>>>(static_cast<const cpx<TS>*>(psi),                 \
-                                         static_cast<cpx<TD>*>(dst), nx, ny, nz, dim, scale)
+  const long long rows_out = (long long)(ny + 1) * (dim == 3 ? nz + 1 : 1);
+#define ROTGP_UP(TS, TD)                                                                       \
+  do {                                                                                         \
+    const bool rows = row_copy<TS, TD>() && nx >= kRowLeast;                                   \
+    const long long work = rows ? (row_tasks(rows_out, nx + 1) + 7) / 8                        \
+                                : (rows_out * (nx + 1) + 255) / 256;                           \
+    auto fn = rows ? k_store<TS, TD, row_copy<TS, TD>()> : k_store<TS, TD, false>;             \
+    fn<<<(int)std::min<long long>(rows ? 152 * 8 : 65536, work), 256, 0, s>>>(                 \
+        static_cast<const cpx<TS>*>(psi), static_cast<cpx<TD>*>(dst), nx, ny, nz, dim, scale); \
+  } while (0)
   if (fp64_store) {
     if (fp64_dst) ROTGP_UP(double, double); else ROTGP_UP(double, float);
   } else {
