@@ -136,6 +136,7 @@ struct rotgp_ctx {
   // default one: weights per axis, points per lane of the rows, own points of
   // the columns' segments (0: not served); dsync for whole blocks of 2D steps
   double2* dtab[3] = {nullptr, nullptr, nullptr};
+  bool dtab_fresh[3] = {false, false, false};
   int d_rows = 0, d_seg[3] = {0, 0, 0};
   dsync* d_sync = nullptr;
   double* partials = nullptr;
@@ -681,8 +682,26 @@ int stencil_weights(rotgp_ctx* c) {
   return ROTGP_OK;
 }
 
-// The tables of one axis and mode: those of the sweeps, of the on-chip
-// stepper and of the complex-double steps.
+// The weights of the complex-double steps of every axis, where they do not match
+// the physics yet: built by the first such step (13 us an axis, which real-time
+// ramps, of Omega step by step, would pay for nothing).  What a capture only
+// records is built again by the next step.
+int double_weights(rotgp_ctx* c) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  for (int a = 0; a < c->grid.dim; ++a) {
+    if (c->dtab_fresh[a]) continue;
+    Timed t(c, K_TABLES);
+    cudaError_t e = cudaStreamIsCapturing(c->stream, &st);
+    if (e == cudaSuccess)
+      e = launch_dtables(c->dtab[a], c->axis[a].nlines, c->halo, c->axis[a].co[1], c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "table kernel");
+    c->dtab_fresh[a] = st == cudaStreamCaptureStatusNone;
+  }
+  return ROTGP_OK;
+}
+
+// The tables of one axis and mode: those of the sweeps and of the on-chip
+// stepper.
 int axis_tables(rotgp_ctx* c, int a, int mode) {
   AxisPlan& ap = c->axis[a];
   ap.co[mode] = make_coef(a, mode, c->grid.h[a], c->phys.dt, c->phys.omega, nlines_u0(c, a),
@@ -694,8 +713,7 @@ int axis_tables(rotgp_ctx* c, int a, int mode) {
     const res_omegas one{{1.0}};
     e = launch_res_tables(c->rtab[a][mode], ap.nlines, c->lt, ap.co[mode], one, 1, c->stream);
   }
-  if (e == cudaSuccess && mode == 1 && c->dtab[a])
-    e = launch_dtables(c->dtab[a], ap.nlines, c->halo, ap.co[mode], c->stream);
+  if (mode == 1) c->dtab_fresh[a] = false;
   return e == cudaSuccess ? ROTGP_OK : cuda_fail(c, e, "table kernel");
 }
 
@@ -1147,8 +1165,12 @@ int run_steps(rotgp_ctx* c, long long n, bool imag) {
   if (!c) return ROTGP_EINVAL;
   if (n < 0) return fail(c, ROTGP_EINVAL, "negative step count");
   if (resident(c, imag) && !one_in_sweeps(c, n, imag)) return resident_steps(c, n, imag, nullptr);
-  if (double_blocks(c, imag)) return double_block(c, n);
   const bool dbl = double_steps(c, imag);
+  if (dbl && n > 0) {
+    const int rc = double_weights(c);
+    if (rc) return rc;
+  }
+  if (double_blocks(c, imag)) return double_block(c, n);
   for (long long s = 0; s < n; ++s) {
     for (int a = 0; a < c->grid.dim; ++a) {
       int rc;

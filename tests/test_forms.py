@@ -68,3 +68,54 @@ def test_calls_of_one_step_take_the_sweeps():
         for _ in range(5):
             s.step_imag(1)
     assert np.array_equal(a.get_psi(), b.get_psi())
+
+
+def test_complex_double_weights_follow_the_physics():
+    """Built by the first imaginary-time step after a change: changes of Omega and
+    Delta between steps, in schedules, in real time and in captured graphs."""
+    from paper_1906_06327_gb300.rotgp import Batch
+    n, h = (48, 40), (0.25, 0.28)
+    a = Solver(n, h, dt=1e-3, precision="fp64", **KW)
+    b = Batch([dict(n=n, h=h, dt=1e-3, **KW)] * 2, precision="fp64")
+    for s in (a, *b.instances):
+        s.init_analytic(1, seed=4)
+        s.step_imag(2)
+        s.set_phys(omega=0.3, dt=8e-4)
+    a.step_imag(3)
+    b.step_imag(3, mode="graph")
+    for s in (a, *b.instances):
+        s.step_schedule(np.array([0.3, 0.25, 0.2]), imag=True)
+        s.step_schedule(np.array([0.2, 0.3]), imag=False)
+        s.set_omega(0.1)
+    a.step_imag(3)
+    b.step_imag(3, mode="graph")
+    a.set_omega(0.4)
+    for s in b.instances:
+        s.set_omega(0.4)
+    a.step_imag(6)
+    b.step_imag(3, mode="graph")
+    b.step_imag(3, mode="graph")
+    t = Solver(n, h, dt=1e-3, precision="fp64", **KW)
+    for ax in (0, 1):
+        t.set_solver(ax, "thomas")
+    t.init_analytic(1, seed=4)
+    t.step_imag(2)
+    t.set_phys(omega=0.3, dt=8e-4)
+    t.step_imag(3)
+    t.step_schedule(np.array([0.3, 0.25, 0.2]), imag=True)
+    t.step_schedule(np.array([0.2, 0.3]), imag=False)
+    t.set_omega(0.1)
+    t.step_imag(3)
+    t.set_omega(0.4)
+    t.step_imag(6)
+    b.sync()
+    ref = t.get_psi()
+    for s in (a, *b.instances):
+        assert np.linalg.norm(s.get_psi() - ref) < 2e-15 * 20 * np.linalg.norm(ref)
+    # real time does not build them: one table launch per axis and mode
+    a.profile(True)
+    a.profile_read()
+    a.set_omega(0.2)
+    a.step_real(1)
+    assert a.profile_read()["tables"]["launches"] == 4
+    b.close()
