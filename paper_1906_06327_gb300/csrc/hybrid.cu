@@ -46,8 +46,12 @@
 
 namespace rotgp {
 
-template <class T, int AX, bool H1, bool IMAG, bool REDUCE>
-__global__ void __launch_bounds__(kHThreads, sizeof(T) == 4 ? 3 : 1) k_line_hybrid(const hybrid_args ha) {
+// MB CTAs per SM: complex float holds 85 registers a thread with three, which pays
+// where there are tiles for them (2048^2 77 us per step against 81 with two), and
+// slows a lone CTA's passes down (512^2 with a halo beyond 64 points 48 against 42,
+// 1501^2 84.7 / 82.9).
+template <class T, int AX, bool H1, bool IMAG, bool REDUCE, int MB>
+__global__ void __launch_bounds__(kHThreads, MB) k_line_hybrid(const hybrid_args ha) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   hybrid_job J;
   J.cs = ha.cs;
@@ -67,7 +71,10 @@ thread_local const char* g_hybrid_stage = "";
 
 template <class T, int AX, bool H1, bool IMAG, bool REDUCE>
 cudaError_t launch_h(const hybrid_args& ha, cudaStream_t s) {
-  auto fn = k_line_hybrid<T, AX, H1, IMAG, REDUCE>;
+  const unsigned blocks = (unsigned)(ha.ngroups * ha.cs);
+  constexpr int few = sizeof(T) == 4 ? 2 : 1, many = sizeof(T) == 4 ? 3 : 1, sms = 152;
+  auto fn = blocks > 2u * sms ? k_line_hybrid<T, AX, H1, IMAG, REDUCE, many>
+                               : k_line_hybrid<T, AX, H1, IMAG, REDUCE, few>;
   const size_t smem = (size_t)kHL * (ha.pc + 4) * sizeof(cpx<T>);
   g_hybrid_stage = "an earlier runtime call";
   cudaError_t e = cudaGetLastError();
@@ -75,7 +82,6 @@ cudaError_t launch_h(const hybrid_args& ha, cudaStream_t s) {
   g_hybrid_stage = "shared-memory opt-in";
   e = allow_smem_bytes((const void*)fn, (int)smem);
   if (e != cudaSuccess) return e;
-  const unsigned blocks = (unsigned)(ha.ngroups * ha.cs);
   if (ha.cs == 1) {
     g_hybrid_stage = "launch";
     fn<<<blocks, kHThreads, smem, s>>>(ha);
@@ -147,11 +153,11 @@ long long hybrid_groups(int axis, long long nlines, int nx) {
 int hybrid_max_clusters(bool fp64, int axis, int cs, int pc) {
   const void* fn = nullptr;
   if (fp64)
-    fn = axis == 0 ? (const void*)k_line_hybrid<double, 0, true, true, false>
-                   : (const void*)k_line_hybrid<double, 1, false, false, true>;
+    fn = axis == 0 ? (const void*)k_line_hybrid<double, 0, true, true, false, 1>
+                   : (const void*)k_line_hybrid<double, 1, false, false, true, 1>;
   else
-    fn = axis == 0 ? (const void*)k_line_hybrid<float, 0, true, true, false>
-                   : (const void*)k_line_hybrid<float, 1, false, false, true>;
+    fn = axis == 0 ? (const void*)k_line_hybrid<float, 0, true, true, false, 2>
+                   : (const void*)k_line_hybrid<float, 1, false, false, true, 2>;
   const size_t smem = hybrid_smem_bytes(pc, fp64);
   cudaError_t e = allow_smem_bytes(fn, (int)smem);
   if (e != cudaSuccess) {
