@@ -53,6 +53,8 @@ struct observe_args {
 void observe_shape(int nx, int ny, int nz, int dim, int sm_count, int* chunk, int* blocks);
 constexpr int kObserveBlocksPerSm = 2;  // most blocks: this times the SMs
 cudaError_t launch_observe(bool fp64, const observe_args& a, int blocks, cudaStream_t s);
+// The vortices in the ellipse that launch_observe left.
+cudaError_t launch_vortex_count(bool fp64, const observe_args& a, cudaStream_t s);
 
 // ABI layout -> device layout, the norm of the loaded state, and from it the
 // pending scale (normalise) or 1; flags bit 0 as the step reductions set it.

@@ -310,8 +310,10 @@ cudaError_t launch_observe(bool fp64, const observe_args& a, int blocks, cudaStr
     else
       k_observe<float, false><<<blocks, 256, 0, s>>>(a);
   }
-  const cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_vortex_count(bool fp64, const observe_args& a, cudaStream_t s) {
   const dim3 grid((unsigned)std::min(16, (a.nx + 255) / 256), (unsigned)std::min(512, a.ny));
   if (fp64)
     k_vort_count<double><<<grid, 256, 0, s>>>(a);

@@ -33,11 +33,11 @@ constexpr int kMaxHalo = 64;
 constexpr int kMaxTable = 512;
 
 enum KernelId {
-  K_SWEEP_X, K_SWEEP_Y, K_SWEEP_Z, K_OBS, K_NORM, K_INIT, K_IO, K_TABLES,
+  K_SWEEP_X, K_SWEEP_Y, K_SWEEP_Z, K_OBS, K_VCOUNT, K_NORM, K_INIT, K_IO, K_TABLES,
   K_XY, K_RESIDENT, K_COUNT
 };
 const char* kKernelNames[K_COUNT] = {"sweep_x_h1",  "sweep_y",        "sweep_z",
-                                     "observables",
+                                     "observables", "vortex_count",
                                      "norm",        "init_analytic",  "pack_unpack",
                                      "tables",      "xy_pass_h1",     "steps_2d"};
 
@@ -1420,6 +1420,10 @@ int ctx_observe(rotgp_ctx* c) {
   {
     Timed t(c, K_OBS);
     e = launch_observe(c->fp64, a, blocks, c->stream);
+  }
+  if (e == cudaSuccess) {
+    Timed t(c, K_VCOUNT);
+    e = launch_vortex_count(c->fp64, a, c->stream);
   }
   if (e != cudaSuccess) return cuda_fail(c, e, "observables kernels");
   e = cudaMemcpyAsync(c->h_obs, c->d_sums(), (OS_COUNT + 1) * sizeof(double),

@@ -119,3 +119,14 @@ def test_complex_double_weights_follow_the_physics():
     a.step_real(1)
     assert a.profile_read()["tables"]["launches"] == 4
     b.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_observables_are_timed_by_kernel(precision):
+    s = Solver((64, 48), (0.2, 0.2), dt=1e-3, precision=precision, **KW)
+    s.init_analytic(1, seed=4)
+    s.profile(True)
+    s.profile_read()
+    s.observables()
+    rec = s.profile_read()
+    assert rec["observables"]["launches"] == 1 and rec["vortex_count"]["launches"] == 1
