@@ -624,7 +624,7 @@ cudaError_t launch_dcols(bool reduce, const dline_args& a, cudaStream_t s) {
 
 bool dstep_fits(int nx, int ny, int halo) {
   const int px = points_per_lane(nx, 4), py = points_per_lane(ny, 4);
-  return px >= 1 && px <= 8 && py >= 1 && py <= 8 && halo <= 32 * std::min(px, py) &&
+  return px >= 1 && px <= 4 && py >= 1 && py <= 8 && halo <= 32 * std::min(px, py) &&
          halo < std::min(nx, ny);
 }
 
@@ -635,7 +635,6 @@ cudaError_t launch_dsteps(const dstep_args& a, int sm_count, cudaStream_t s) {
     case 1: return launch_2d<1>(a, py, blocks, s);
     case 2: return launch_2d<2>(a, py, blocks, s);
     case 4: return launch_2d<4>(a, py, blocks, s);
-    case 8: return launch_2d<8>(a, py, blocks, s);
   }
   return cudaErrorInvalidValue;
 }

@@ -35,10 +35,12 @@ struct dline_args {
   const double* scale;
 };
 
-// Rows (x sweep with H1): points per lane for lines of N points, 0 if none.
+// Rows (x sweep with H1): points per lane for lines of N points, at most 16 (512
+// points); 0 if none.
 int drow_points(int N, int halo);
 cudaError_t launch_drows(const dline_args& a, int P, cudaStream_t s);
-// Columns (y and z sweeps): own points of a segment, and the blocks.
+// Columns (y and z sweeps): own points of a segment (0: none, lines of more than
+// 96 points with a halo above 48), and the blocks.
 int dcol_segment(int N, long long lines, int halo, int sm_count);
 long long dcol_blocks(int nx, long long lines, int len, int seg);
 cudaError_t launch_dcols(bool reduce, const dline_args& a, cudaStream_t s);
@@ -59,7 +61,7 @@ struct dstep_args {
   int* flags;
   dsync* sync;
 };
-// Can lines of nx and ny points with this halo run there?
+// Can lines of nx (at most 512) and ny (1,024) points with this halo run there?
 bool dstep_fits(int nx, int ny, int halo);
 cudaError_t launch_dsteps(const dstep_args& a, int sm_count, cudaStream_t s);
 

@@ -287,7 +287,7 @@ bool tail_plan(int axis, int N, int nx, long long lines, int halo, bool imag, si
   const int H = std::max(1, halo - 2);
   // long tails are run over more own points
   int L = H > 12 ? 32 : 16;
-  if (axis == 0 && !imag) L = 16;
+  if (axis == 0 && !imag) L = 16;  // (the rest of H1 takes the room)
   const int tiles = (N + kTailWarps * L - 1) / (kTailWarps * L);
   s->L = L;
   s->nw = std::min(kTailWarps, (N + tiles * L - 1) / (tiles * L));
@@ -300,8 +300,7 @@ bool tail_plan(int axis, int N, int nx, long long lines, int halo, bool imag, si
 }
 
 cudaError_t launch_tail_x(bool imag, const tail_args& a, cudaStream_t s) {
-  auto fn = a.sh.L == 32 ? (imag ? k_tail_x<32, true> : k_tail_x<32, false>)
-                         : (imag ? k_tail_x<16, true> : k_tail_x<16, false>);
+  auto fn = !imag ? k_tail_x<16, false> : a.sh.L == 32 ? k_tail_x<32, true> : k_tail_x<16, true>;
   const cudaError_t e = allow_smem_bytes((const void*)fn, (int)a.sh.smem);
   if (e != cudaSuccess) return e;
   fn<<<(unsigned)a.sh.blocks, 32 * a.sh.nw, a.sh.smem, s>>>(a);
