@@ -49,7 +49,8 @@ extern "C" {
 #define ROTGP_ETIMEOUT (-6)     /* a bounded device wait (TMA load) ran out  */
 
 #define ROTGP_FP64 0 /* complex double throughout                           */
-#define ROTGP_FP32 1 /* complex float bulk; norm, energy, mu, rms in double  */
+#define ROTGP_FP32 1 /* complex float bulk; norm, energy, mu, rms summed in
+                        float pairs (48 bits) per block, then in double     */
 
 typedef struct rotgp_ctx rotgp_ctx;
 
@@ -193,10 +194,13 @@ int rotgp_column_density(rotgp_ctx* ctx, double* dst, int dst_on_device);
 /* Enqueue n split steps in imaginary time (i Delta -> Delta, then
  * renormalisation) or in real time.  n >= 0.  Eq. split with the substeps
  * of Eqs. eq1-eq3 (and z in 3D), each line solved as in Eqs. eqD.9-eqD.11.
- * Real time in complex float keeps the norm to about 1e-12 to 3e-10 per
- * step (the CN map and the H1 rotation are unitary in exact arithmetic;
- * the kernels order their float arithmetic so that rounding adds no
- * systematic gain); in complex double to 1e-16. */
+ * The CN map and the H1 rotation are unitary in exact arithmetic.  In complex
+ * float the line weights are rounded, which moves the norm of a smooth state
+ * by about 8e-7 kappa^2 per step and axis, kappa = Delta / (4 h^2), of either
+ * sign, the same every step (1e-12 at kappa = 0.001, 5e-10 at 0.025, 8e-9 at
+ * 0.1; at single kappas up to eight times that); the kernels order their
+ * arithmetic so that rounding the state adds no systematic gain.  In complex
+ * double the norm stays to 1e-16. */
 int rotgp_step_imag(rotgp_ctx* ctx, long long n);
 int rotgp_step_real(rotgp_ctx* ctx, long long n);
 
@@ -232,13 +236,15 @@ int rotgp_info(const rotgp_ctx* ctx, rotgp_solver_info* out);
  * block, taking 32-line units round-robin) and
  * segments each line is split into (clamped to the number of chunks).
  * The one-line-per-thread TMA forms (chunk 8 or 16) solve the unfolded
- * system psi' = 2 A^-1 psi - psi, in real time centred about psi so that its
- * rounded weights keep the CN map's norm; an axis with Delta / (4 h^2) above
- * 0.005 runs its real-time steps in the default two-lines-per-thread form.  Changes speed only: every shape
- * gives results equal up to the truncation bound of the chunked line solver.
- * Used by the autotuner.  On an axis in the exact partition solve (ROTGP_SOLVER_HYBRID)
- * only `segments` applies: the number of CTAs (1, 2, 4 or 8, one cluster)
- * that share each line; results are equal up to rounding.
+ * system psi' = 2 A^-1 psi - psi, in real time centred about psi (weights of
+ * the order of kappa); an axis with Delta / (4 h^2) above 0.005 runs its
+ * real-time steps in the default two-lines-per-thread form.  Changes speed
+ * only: every shape gives results equal up to the truncation bound of the
+ * chunked line solver.  Used by the autotuner.  On an axis in the exact
+ * partition solve (ROTGP_SOLVER_HYBRID, or the default with a halo above 16
+ * points) only `segments` applies, and selects that solve: the number of CTAs
+ * (1, 2, 4 or 8, one cluster) that share each line; results are equal up to
+ * rounding.
  * ROTGP_EINVAL for a shape that is not built or does not fit. */
 int rotgp_tune(rotgp_ctx* ctx, int axis, int lines_per_lane, int chunk, int ring,
                int warps_per_block, int segments);
@@ -261,11 +267,12 @@ int rotgp_tune(rotgp_ctx* ctx, int axis, int lines_per_lane, int chunk, int ring
  * steps always use the Thomas form, whose Crank-Nicolson map stays unitary
  * with rounded coefficients (independently rounded stencil weights would
  * let the norm drift by ~1e-7 per step in float).
- * ROTGP_SOLVER_HYBRID: the same Thomas solution of every whole line with
- *   nothing truncated, by a partition method: each line is cut into
- *   segments that run the Thomas recurrences locally from zero carries, the
- *   true carries follow from composing the segments' affine summaries (the
- *   reduced system), and the segments rerun from them.  A line lives in the
+ * ROTGP_SOLVER_HYBRID: the same Thomas solution of every whole line up to
+ *   rounding, by a partition method: each line is cut into segments that run
+ *   the Thomas recurrences locally from zero carries, the true carries follow
+ *   from composing the segments' affine summaries (the reduced system), and
+ *   each segment adds what its true carry adds to it, down to 1e-10 of the
+ *   carry in float and 1e-19 in double.  A line lives in the
  *   shared memory of one CTA or of a cluster of up to 8 CTAs (distributed
  *   shared memory), so each point is read and written once per sweep;
  *   complex float and double, both propagation modes.  It serves long lines
@@ -285,13 +292,15 @@ int rotgp_tune(rotgp_ctx* ctx, int axis, int lines_per_lane, int chunk, int ring
  * (A call of a single imaginary-time step runs in the sweeps where those are
  * the faster ones: even N_x and a halo of at most 8 points.)
  * A wait between its tiles is bounded (about 2 s of device time,
- * ROTGP_ETIMEOUT).  Likewise imaginary-time steps in complex double with a
- * halo of at most 64 points, shorter than the lines, run in kernels of their
- * own (records "steps_2d" for whole blocks of 2D steps of lines up to 1024
- * points, else the sweeps' names), equal to the sweeps up to rounding; and
- * complex-float sweeps with a halo of 17 to 64 points, or with odd N_x, take
- * truncated tiles of lines instead of the forms named above, with results
- * equal up to rounding and the truncation bound.
+ * ROTGP_ETIMEOUT).  Likewise imaginary-time steps in complex double with N_x
+ * up to 512 and a halo shorter than the lines, of at most 48 points (64 where
+ * N_y and N_z are at most 96), run in kernels of their own (records "steps_2d"
+ * for whole blocks of 2D steps with N_y up to 1,024, else the sweeps' names),
+ * equal to the sweeps up to rounding; and complex-float sweeps with odd N_x, or
+ * with a halo of 17 to 64 points on lines of at least 2 halo + 32 points or
+ * where there are at least 8,192 of them, take truncated tiles of lines instead
+ * of the forms named above, with results equal up to rounding and the
+ * truncation bound.
  * The y and z sweeps in stencil form, and the fused pass, stage their
  * tiles with TMA loads whose waits are bounded: a wait that runs out
  * (about 2 s) makes the next synchronising call return ROTGP_ETIMEOUT. */
@@ -306,14 +315,15 @@ int rotgp_set_solver(rotgp_ctx* ctx, int axis, int solver);
  * per axis that the context supports, and the fused x-y pass with each form
  * of the z sweep; then, for the chosen forms, the lines per lane, chunk
  * length and segment count of each Thomas sweep together, its ring depth,
- * and the segment count of each stencil y/z sweep (as rotgp_tune).  Each candidate runs one warm-up step
- * and then twice `steps` imaginary-time steps from a copy of the current
- * state, timed with CUDA events on the context's stream (the faster repeat
- * counts), and so does the on-chip 2D stepper where the context has one
- * (selected, it shows as THOMAS on both axes); the state, its pending
+ * and the segment count of each stencil y/z sweep (as rotgp_tune).  Each
+ * candidate runs one warm-up step and then twice `steps` imaginary-time steps
+ * from a copy of the current state, timed with CUDA events on the context's
+ * stream (the faster repeat counts), and so does the default plan where it has
+ * kernels of its own (rotgp_set_solver), with the forms and shapes from before
+ * the call, which stay with it (selected, *choice is 0); the state, its pending
  * renormalisation and the step counter are restored afterwards, and the
- * fastest candidate stays selected.  *choice (if not NULL) receives it as a bit set: bit a =
- * axis a in stencil form, bit 3 = fused x-y pass, bit 4 + a = axis a in the
+ * fastest candidate stays selected.  *choice (if not NULL) receives it as a bit
+ * set: bit a = axis a in stencil form, bit 3 = fused x-y pass, bit 4 + a = axis a in the
  * exact partition solve (candidates include every supported combination
  * with it).  Synchronises the stream.
  * ROTGP_EINVAL if steps < 1. */

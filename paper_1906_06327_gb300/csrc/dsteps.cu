@@ -30,9 +30,9 @@
 // with its halos.  H1: the exponential is a Taylor series of degree 9 where
 // the step's exponent is below 1/16.
 //
-// A small 2D state runs a whole block of steps in one cooperative launch, a
-// line at a time on all four schedulers of an SM, with a grid-wide exchange
-// after each sweep (one 64-bit word pair that takes every CTA's count and
+// A 2D state (of up to 512 points in x, 1,024 in y) runs a whole block of steps in one
+// cooperative launch, a line at a time on all four schedulers of an SM, with a
+// grid-wide exchange after each sweep (one 64-bit word pair that takes every CTA's count and
 // share of the norm, as in resident.cu, here in 85-bit integers).
 //
 // GB300, before / after: 128^2 step 134 / 11.9 us; 256 x 256 x 32 step 1,120 /

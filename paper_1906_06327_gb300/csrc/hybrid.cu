@@ -1,4 +1,4 @@
-// hybrid.cu -- exact line solves of one Crank-Nicolson sweep (Sec. 2, the
+// hybrid.cu -- whole-line solves of one Crank-Nicolson sweep (Sec. 2, the
 // tridiagonal systems of Eqs. eqD.11/eq5) by a partition method, for lines
 // that the chunked solver of sweep_x.cu / sweep_s.cu serves badly or not at
 // all: long lines whose Thomas carries decay slowly (Delta/h^2 large, so the
@@ -17,10 +17,11 @@
 // (backward), which is the reduced system of the partition method, solved
 // here by direct composition; the segments then add what the true carry adds
 // to their local solution, the products of the multipliers times it, over the
-// points in which that is above a thousandth of the rounding (rerunning both
-// recurrences from the true carries, as before, doubled the instructions: a
-// 4096^2 step 411 / 307 us, a step of the 64-instance batch 196 / 173 us).  Nothing is truncated: the result is the Thomas solution
-// of the whole line up to rounding, whatever the decay of the carries.
+// points in which that is above a thousandth of the rounding (1e-10 of the carry
+// in float, 1e-19 in double; rerunning both recurrences from the true carries, as
+// before, doubled the instructions: a 4096^2 step 411 / 307 us, a step of the
+// 64-instance batch 196 / 173 us).  No halo is cut off: whatever the decay of
+// the carries, the result is the Thomas solution of the whole line up to rounding.
 //
 // Layout.  A CTA of 256 threads holds a tile of 16 lines x pc positions (+2
 // halo positions either side) in shared memory; thread (line l, sub-segment

@@ -1018,12 +1018,15 @@ int tail_step(rotgp_ctx* c, int axis, bool imag, bool last) {
   return ROTGP_OK;
 }
 
-// May real time take the centred TMA sweeps on this axis?  Their weights m2 - 2,
-// al and be, of size up to 4 kappa, are rounded one by one, which moves the norm
-// by up to 1e-6 kappa^2 per step, the same way every step (measured 1.8e-9 at
-// kappa_z = 0.04, where the folded form moves it by 3e-10).  Up to 0.005 that is
-// 2.5e-11 per axis, within what the folded form itself does; 256 x 256 x 128 at
-// kappa 0.004 takes 87.5 us per step there, 128 folded.
+// May real time take the centred TMA sweeps on this axis?  Weights rounded to float
+// move the norm of a smooth state by about 8e-7 kappa^2 per step and axis, of
+// either sign and at single kappas up to eight times that, in the centred, the
+// folded and the two-tail form alike (tests/test_norm_weights.py): which one does
+// better at a given kappa is chance (0.04: centred -1.8e-9, folded 3e-10; 0.06: 1.8e-9
+// and -4.7e-9).  Up to 0.005 the gain is below 6e-11 in each, and the centred sweeps
+// are the faster ones (256 x 256 x 128 at kappa 0.004 87.5 us per step, 128 folded);
+// beyond, real time keeps the folded form, in which the long runs are pinned (the
+// 256 x 256 x 32 disk, kappa_z = 0.04).
 bool centred_ok(const rotgp_ctx* c, int axis) {
   const double h = c->grid.h[axis];
   return 0.25 * std::fabs(c->phys.dt) <= 0.005 * h * h;
@@ -1175,10 +1178,10 @@ int run_steps(rotgp_ctx* c, long long n, bool imag) {
     for (int a = 0; a < c->grid.dim; ++a) {
       int rc;
       // the stencil and fused forms serve imaginary time; real-time steps
-      // keep Thomas forms whose near-unit factors are stored as their
-      // difference from 1 or 2, so that the rounded CN map stays unitary to
-      // ~1e-10 per sweep (the stencil's rounded central weight, close to 1
-      // itself, would not)
+      // keep forms whose near-unit factors are stored as their difference from
+      // 1 or 2, so that the rounded CN map stays unitary to some 1e-6 kappa^2
+      // per sweep (the stencil's rounded central weight, close to 1 itself,
+      // would not)
       if (a == 0 && c->fuse_xy && imag) {
         rc = xy_pass(c, imag);
         ++a;  // the y sweep is part of the pass

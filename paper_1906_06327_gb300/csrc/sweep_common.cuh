@@ -30,7 +30,8 @@
 // points), TMA box loads and stores through R + 1 slots per warp, persistent
 // warps and programmatic launch; real time solves it in the centred form
 // (weight m2 - 2, see k_sweep_s1t) where kappa is small, and the folded form
-// above elsewhere, each holding the CN map's norm to rounding.
+// above elsewhere, each holding the CN map's norm to the rounding of weights of
+// the order of kappa.
 #pragma once
 
 #include "common.cuh"

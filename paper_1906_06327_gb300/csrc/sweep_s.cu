@@ -521,9 +521,9 @@ static cudaError_t dispatch_s2(bool reduce, const stream_args& a, const sweep_sh
 // of the order of kappa (mc = m2 - 2 in the first plane): t_p = d_p - 2 psi_p =
 // mc psi_p + al d_{p-1}, psi'_p = psi_p + (t_p + be z_{p+1}).  The plain form
 // doubles the rounding of m2 every step, which moves the real-time norm by
-// 2e-4 per time unit; this one by at most 1e-6 kappa^2 per step, and serves axes
-// up to kappa = 0.005, at two more operations a point instead of four
-// more complex products (GB300, 256 x 256 x 128 real-time step 128 us in the
+// 2e-4 per time unit; this one, like the folded form, by about 8e-7 kappa^2 per
+// step, and it serves axes up to kappa = 0.005 (rotgp.cu), at two more
+// operations a point instead of four more complex products (GB300, 256 x 256 x 128 real-time step 128 us in the
 // folded sweeps, 87.5 in these).
 template <int C, bool REDUCE, int RING, int AX, bool CEN>
 __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_s1t(const __grid_constant__ CUtensorMap map,
