@@ -146,6 +146,15 @@ cudaError_t after_resident(rotgp_batch* b, int i, bool imag, int* before) {
   return e;
 }
 
+// Later work of the instances on their own streams (their steps, observables, I/O)
+// follows what was launched on the batch's stream.
+int release_streams(rotgp_batch* b, const std::vector<int>& set) {
+  cudaError_t e = cudaEventRecord(b->fork, b->stream);
+  for (size_t k = 0; k < set.size() && e == cudaSuccess; ++k)
+    e = cudaStreamWaitEvent(b->streams[set[k]], b->fork, 0);
+  return e == cudaSuccess ? ROTGP_OK : bfail(b, ROTGP_ECUDA, "order: %s", cudaGetErrorString(e));
+}
+
 int run_set_inner(rotgp_batch* b, const std::vector<int>& set, long long n, bool imag,
                   int mode) {
   cudaError_t e;
@@ -172,13 +181,7 @@ int run_set_inner(rotgp_batch* b, const std::vector<int>& set, long long n, bool
     if (e != cudaSuccess)
       return bfail(b, ROTGP_ECUDA, "persistent batch launch: %s", cudaGetErrorString(e));
     for (int i : set) rotgp::ctx_add_steps(b->ctx[i], n);
-    // later work of the instances (observables, I/O) follows the launch
-    if ((e = cudaEventRecord(b->fork, b->stream)) != cudaSuccess)
-      return bfail(b, ROTGP_ECUDA, "order: %s", cudaGetErrorString(e));
-    for (int i : set)
-      if ((e = cudaStreamWaitEvent(b->streams[i], b->fork, 0)) != cudaSuccess)
-        return bfail(b, ROTGP_ECUDA, "order: %s", cudaGetErrorString(e));
-    return ROTGP_OK;
+    return release_streams(b, set);
   }
   if (mode != ROTGP_BATCH_GRAPH) {
     if ((e = cudaEventRecord(b->fork, b->stream)) != cudaSuccess)
@@ -263,7 +266,7 @@ int run_set_inner(rotgp_batch* b, const std::vector<int>& set, long long n, bool
   if ((e = cudaGraphLaunch(g->exec, b->stream)) != cudaSuccess)
     return bfail(b, ROTGP_ECUDA, "graph launch: %s", cudaGetErrorString(e));
   ++b->graph_launches;
-  return ROTGP_OK;
+  return release_streams(b, set);
 }
 
 }  // namespace

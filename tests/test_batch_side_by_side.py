@@ -77,3 +77,31 @@ def test_a_graph_of_many_is_not_one_after_another(n, count, precision):
             best[mode] = min(best.get(mode, 1e9), time.perf_counter() - t)
     b.close()
     assert best["graph"] < 0.7 * best["direct"], best
+
+
+@pytest.mark.parametrize("mode", ["graph", "direct", "persistent"])
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_instances_follow_the_batch(mode, precision):
+    """An instance read or stepped by itself right after a block of batch steps, with
+    nothing waited for in between."""
+    specs = _specs((128, 96), 6)
+    got = []
+    for wait in (True, False):
+        b = Batch(specs, precision=precision)
+        for i, s in enumerate(b.instances):
+            s.init_analytic(1, seed=i)
+        for _ in range(3):
+            b.step_imag(150, mode=mode)
+            if wait:
+                b.sync()
+        first = b.instances[5].get_psi()
+        b.instances[4].step_real(3)
+        b.step_imag(150, mode=mode)
+        if wait:
+            b.sync()
+        b.instances[3].set_omega(0.4)
+        b.instances[3].step_imag(4)
+        got.append([first] + [s.get_psi() for s in b.instances])
+        b.close()
+    for x, y in zip(*got):
+        assert np.array_equal(x, y)
