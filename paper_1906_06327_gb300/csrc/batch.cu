@@ -161,6 +161,8 @@ int run_set_inner(rotgp_batch* b, const std::vector<int>& set, long long n, bool
   // work already queued on the instance streams (table rebuilds of
   // rotgp_set_phys, state I/O) comes first
   for (int i : set) {
+    const int rc = mode == ROTGP_BATCH_PERSISTENT ? ROTGP_OK : rotgp::ctx_prepare(b->ctx[i], imag);
+    if (rc) return bfail(b, rc, "instance %d: %s", i, rotgp_last_error(b->ctx[i]));
     if ((e = cudaEventRecord(b->done[i], b->streams[i])) != cudaSuccess ||
         (e = cudaStreamWaitEvent(b->stream, b->done[i], 0)) != cudaSuccess)
       return bfail(b, ROTGP_ECUDA, "order: %s", cudaGetErrorString(e));

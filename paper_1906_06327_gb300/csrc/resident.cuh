@@ -78,6 +78,8 @@ struct ctx_cost {
   double alone, beside, least;
 };
 ctx_cost ctx_step_cost(const rotgp_ctx* c, bool imag, long long n);
+// Build what steps of this mode would build first (a capture would record it).
+int ctx_prepare(rotgp_ctx* c, bool imag);
 // Steps from here on beside other instances' (no launch over the whole chip).
 void ctx_set_beside(rotgp_ctx* c, bool on);
 // Points over which a line carry of the context stays above the rounding of

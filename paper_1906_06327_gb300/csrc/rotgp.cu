@@ -1335,6 +1335,7 @@ int ctx_carry_reach(const rotgp_ctx* c) {
 bool ctx_resident(const rotgp_ctx* c, bool imag) {
   return resident(c, imag) || double_blocks(c, imag);
 }
+int ctx_prepare(rotgp_ctx* c, bool imag) { return double_steps(c, imag) ? double_weights(c) : ROTGP_OK; }
 void ctx_set_beside(rotgp_ctx* c, bool on) { c->beside = on; }
 ctx_cost ctx_step_cost(const rotgp_ctx* c, bool imag, long long n) {
   // Microseconds on GB300: straight lines through graphs of 2 to 64 instances of
