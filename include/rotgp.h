@@ -199,8 +199,8 @@ int rotgp_column_density(rotgp_ctx* ctx, double* dst, int dst_on_device);
  * by about 8e-7 kappa^2 per step and axis, kappa = Delta / (4 h^2), of either
  * sign, the same every step (1e-12 at kappa = 0.001, 5e-10 at 0.025, 8e-9 at
  * 0.1, 1e-7 to 3e-7 from 0.3 on; at single kappas up to eight times that); the
- * kernels order their arithmetic so that rounding the state adds no systematic
- * gain.  In complex double the norm stays to 1e-16. */
+ * kernels order their arithmetic, and round small changes up or down without
+ * bias, so that rounding the state adds no systematic gain.  In complex double the norm stays to 1e-16. */
 int rotgp_step_imag(rotgp_ctx* ctx, long long n);
 int rotgp_step_real(rotgp_ctx* ctx, long long n);
 

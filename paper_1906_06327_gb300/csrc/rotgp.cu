@@ -960,7 +960,7 @@ int xy_pass(rotgp_ctx* c, bool imag) {
 // partition solve), and rows that are not 16-byte multiples, which the TMA
 // sweeps cannot read (255 x 256 x 128 167 us against 194 in imaginary time, 171
 // against 233 in real time; 65 x 49 x 33 27 against 36).  On even rows the TMA
-// sweeps are the faster ones (256 x 256 x 128 67 us in imaginary and 87 us in
+// sweeps are the faster ones (256 x 256 x 128 67 us in imaginary and 99 us in
 // real time, against 145 in tiles).  Short lines with a halo above 16 stay in the
 // exact partition solve as long as one wave of its tiles takes them all: a tile
 // of tails runs H + L points in sequence whatever the length, a thread of the
@@ -1024,7 +1024,7 @@ int tail_step(rotgp_ctx* c, int axis, bool imag, bool last) {
 // folded and the two-tail form alike (tests/test_norm_weights.py): which one does
 // better at a given kappa is chance (0.04: centred -1.8e-9, folded 3e-10; 0.06: 1.8e-9
 // and -4.7e-9).  Up to 0.005 the gain is below 6e-11 in each, and the centred sweeps
-// are the faster ones (256 x 256 x 128 at kappa 0.004 87.5 us per step, 128 folded);
+// are the faster ones (256 x 256 x 128 at kappa 0.004 99 us per step, 128 folded);
 // beyond, real time keeps the folded form, in which the long runs are pinned (the
 // 256 x 256 x 32 disk, kappa_z = 0.04).
 bool centred_ok(const rotgp_ctx* c, int axis) {

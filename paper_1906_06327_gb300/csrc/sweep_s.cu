@@ -523,8 +523,8 @@ static cudaError_t dispatch_s2(bool reduce, const stream_args& a, const sweep_sh
 // doubles the rounding of m2 every step, which moves the real-time norm by
 // 2e-4 per time unit; this one, like the folded form, by about 8e-7 kappa^2 per
 // step, and it serves axes up to kappa = 0.005 (rotgp.cu), at two more
-// operations a point instead of four more complex products (GB300, 256 x 256 x 128 real-time step 128 us in the
-// folded sweeps, 87.5 in these).
+// operations a point instead of four more complex products and the dithered sum (GB300, 256 x 256 x 128 real-time step
+// 128 us in the folded sweeps, 99 in these; 87.5 with sums rounded to nearest).
 template <int C, bool REDUCE, int RING, int AX, bool CEN>
 __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_s1t(const __grid_constant__ CUtensorMap map,
                                                    const __grid_constant__ CUtensorMap omap,
@@ -691,7 +691,7 @@ __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_s1t(const __grid_c
           for (int r = C - 1; r >= 0; --r) {
             z = bstep(BER, BEI, z, prv[r]);
             const float2 v = sp[r * 32];
-            const float2 o = CEN ? __fadd2_rn(v, z) : __ffma2_rn(NEG1, v, z);
+            const float2 o = CEN ? add_dithered(v, z) : __ffma2_rn(NEG1, v, z);
             if (CEN) z = twice(v, z);
             sp[r * 32] = o;
             if (REDUCE) n2 = __ffma2_rn(o, o, n2);
@@ -706,7 +706,7 @@ __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_s1t(const __grid_c
               wsplit(kb[r], br, bi);
               z = bstep(br, bi, z, prv[r]);
               const float2 v = sp[r * 32];
-              const float2 o = CEN ? __fadd2_rn(v, z) : __ffma2_rn(NEG1, v, z);
+              const float2 o = CEN ? add_dithered(v, z) : __ffma2_rn(NEG1, v, z);
               if (CEN) z = twice(v, z);
               sp[r * 32] = o;
               if (REDUCE) n2 = __ffma2_rn(o, o, n2);

@@ -785,7 +785,7 @@ __global__ void __launch_bounds__(C == 8 ? 512 : 256) k_sweep_x1t(const __grid_c
         const float2* rq = rest + (qq & 1) * SLOT;
         auto result = [&](float2 psi, int r) -> float2 {
           if (IMAG) return __ffma2_rn(NEG1, psi, z);
-          const float2 o = __fadd2_rn(psi, __fadd2_rn(rq[r * 32], z));
+          const float2 o = add_dithered(psi, __fadd2_rn(rq[r * 32], z));
           z = twice(psi, z);
           return o;
         };

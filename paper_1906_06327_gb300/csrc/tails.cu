@@ -19,6 +19,7 @@
 // passes trimmed); 255 x 256 x 128 imaginary time x 74 / 55, y 57 / 54, z 66 / 64
 // us, real time x 113 / 60 us.
 #include <algorithm>
+#include <type_traits>
 
 #include "pairsum.cuh"
 #include "tail_solve.cuh"
@@ -114,7 +115,7 @@ __device__ __forceinline__ void tail_norm(fpair v, const tail_args& a) {
 }
 
 // ---------------------------------------------------------------- columns
-template <int L, bool REDUCE>
+template <int L, bool REDUCE, bool IMAG>
 __global__ void __launch_bounds__(32 * kTailWarps, 2) k_tail_s(const tail_args a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* T = reinterpret_cast<float2*>(smem_raw);  // [point][lane]
@@ -163,8 +164,8 @@ __global__ void __launch_bounds__(32 * kTailWarps, 2) k_tail_s(const tail_args a
     int left;     // own positions inside the line
     bool act, edge;
     __device__ __forceinline__ float2 operator()(int i, float2 w, float2 c) {
-      const float2 o = make_float2(w.x + c.x, w.y + c.y);
-      return i == 0 && edge ? make_float2(0.f, 0.f) : o;
+      if (i == 0 && edge) return make_float2(0.f, 0.f);
+      return IMAG ? make_float2(w.x + c.x, w.y + c.y) : add_dithered(w, c);
     }
     __device__ __forceinline__ void done(const float2 (&o)[L]) {
 #pragma unroll
@@ -258,7 +259,8 @@ __global__ void __launch_bounds__(32 * kTailWarps, 2) k_tail_x(const tail_args a
     bool edge;
     __device__ __forceinline__ float2 operator()(int i, float2 w, float2 c) {
       if (!IMAG) c = make_float2(c.x + rest[i].x, c.y + rest[i].y);
-      return i == 0 && edge ? make_float2(0.f, 0.f) : make_float2(w.x + c.x, w.y + c.y);
+      if (i == 0 && edge) return make_float2(0.f, 0.f);
+      return IMAG ? make_float2(w.x + c.x, w.y + c.y) : add_dithered(w, c);
     }
     __device__ __forceinline__ void done(const float2 (&r)[L]) {
       // every warp has read its neighbours' points: the results take their place
@@ -308,8 +310,12 @@ cudaError_t launch_tail_x(bool imag, const tail_args& a, cudaStream_t s) {
 }
 
 cudaError_t launch_tail_s(bool reduce, const tail_args& a, cudaStream_t s) {
-  auto fn = a.sh.L == 32 ? (reduce ? k_tail_s<32, true> : k_tail_s<32, false>)
-                         : (reduce ? k_tail_s<16, true> : k_tail_s<16, false>);
+  auto pick = [&](auto im) {
+    constexpr bool IMAG = decltype(im)::value;
+    return a.sh.L == 32 ? (reduce ? k_tail_s<32, true, IMAG> : k_tail_s<32, false, IMAG>)
+                        : (reduce ? k_tail_s<16, true, IMAG> : k_tail_s<16, false, IMAG>);
+  };
+  auto fn = a.imag ? pick(std::true_type{}) : pick(std::false_type{});
   const cudaError_t e = allow_smem_bytes((const void*)fn, (int)a.sh.smem);
   if (e != cudaSuccess) return e;
   fn<<<(unsigned)a.sh.blocks, 32 * a.sh.nw, a.sh.smem, s>>>(a);
