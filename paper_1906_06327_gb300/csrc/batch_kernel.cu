@@ -171,6 +171,7 @@ __global__ void __launch_bounds__(kHThreads, sizeof(T) == 4 ? 3 : 1) k_batch_ste
       a.out = I.psi[1 - I.cur];
       a.coef = I.tab[0][IMAG ? 1 : 0];
       a.len = I.nx;
+      a.imag = IMAG;
       a.halo = I.reach;
       a.lt = I.lt;
       a.nlines = I.ny;
@@ -209,6 +210,7 @@ __global__ void __launch_bounds__(kHThreads, sizeof(T) == 4 ? 3 : 1) k_batch_ste
       a.out = I.psi[I.cur];
       a.coef = I.tab[1][IMAG ? 1 : 0];
       a.len = I.ny;
+      a.imag = IMAG;
       a.halo = I.reach;
       a.lt = I.lt;
       a.nlines = I.nx;

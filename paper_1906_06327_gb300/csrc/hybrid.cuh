@@ -100,6 +100,16 @@ struct int_tag {
   static constexpr int value = V;
 };
 
+// A value and what its true carry adds to it.
+template <bool DITHER, class T>
+__device__ __forceinline__ cpx<T> joined(cpx<T> p, cpx<T> q) {
+  if constexpr (DITHER && sizeof(T) == 4) {
+    const float2 r = add_dithered(make_float2(p.x, p.y), make_float2(q.x, q.y));
+    return mk<T>(r.x, r.y);
+  }
+  return p + q;
+}
+
 template <class T, int AX, bool H1, bool IMAG, bool REDUCE>
 __device__ __forceinline__ double hybrid_tile(const stream_args& a, const hybrid_job& J,
                                               unsigned char* smem_raw) {
@@ -322,21 +332,30 @@ __device__ __forceinline__ double hybrid_tile(const stream_args& a, const hybrid
   __syncthreads();
 
   // ---- the true carry: d_p += (product of al) carry over the `reach` points
-  // in which it is above rounding
-  {
+  // in which it is above rounding.  A carry below half a unit of the last place
+  // of d_p would be lost every time: in real time the sums are rounded up or down
+  // instead so that none of it is on average (add_dithered; norm per step of 128^2,
+  // kappa 0.01 and 0.05, -8e-9 and 1.2e-8 without, 2e-10 and 2e-9 with it, as with
+  // recurrences rerun from their carries).
+  const bool dither = sizeof(T) == 4 && !a.imag;
+  auto forward = [&](auto tag) {
     E c = sD[l][k];
     const int n = min(nv, reach);
     int i = 0;
     for (; i < min(n, it); ++i) {
       c = cmul(crow[pb + i].al, c);
-      el(l, eb + i) = el(l, eb + i) + c;
+      el(l, eb + i) = joined<decltype(tag)::value != 0>(el(l, eb + i), c);
     }
 #pragma unroll 4
     for (; i < n; ++i) {
       c = cmul(cinf.al, c);
-      el(l, eb + i) = el(l, eb + i) + c;
+      el(l, eb + i) = joined<decltype(tag)::value != 0>(el(l, eb + i), c);
     }
-  }
+  };
+  if (dither)
+    forward(int_tag<1>{});
+  else
+    forward(int_tag<0>{});
   // ---- backward from a zero carry, x over d; summary (prod be, x at the start)
   {
     E x = zero<T>(), B = mk<T>(1, 0);
@@ -395,20 +414,24 @@ __device__ __forceinline__ double hybrid_tile(const stream_args& a, const hybrid
   csync();
 
   // ---- the true carry: x_p += (product of be) carry, from the end
-  {
+  auto backward = [&](auto tag) {
     E c = sD[l][k];
     const int n0 = max(0, nv - reach);
     int i = nv - 1;
 #pragma unroll 4
     for (; i >= max(n0, it); --i) {
       c = cmul(cinf.be, c);
-      el(l, eb + i) = el(l, eb + i) + c;
+      el(l, eb + i) = joined<decltype(tag)::value != 0>(el(l, eb + i), c);
     }
     for (; i >= n0; --i) {
       c = cmul(crow[pb + i].be, c);
-      el(l, eb + i) = el(l, eb + i) + c;
+      el(l, eb + i) = joined<decltype(tag)::value != 0>(el(l, eb + i), c);
     }
-  }
+  };
+  if (dither)
+    backward(int_tag<1>{});
+  else
+    backward(int_tag<0>{});
   __syncthreads();
   acc_t<T> acc;
 

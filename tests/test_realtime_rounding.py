@@ -39,3 +39,22 @@ def test_small_changes_are_rounded_without_bias(n, form, kappa):
     t.step_real(STEPS)
     ref = t.get_psi()
     assert np.linalg.norm(s.get_psi() - ref) < 5e-6 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("n,kappa,per_step", [((128, 128), 0.0005, 4e-10),
+                                              ((128, 128), 0.01, 1.3e-9),
+                                              ((256, 256), 0.01, 1.3e-9)])
+@pytest.mark.parametrize("omega", [0.0, 0.7])
+def test_exact_solve_joins_its_carries_without_bias(n, kappa, per_step, omega):
+    """Carries below half a unit of the last place are not lost.  Bounds: as above, or
+    eight times the rms effect of rounded weights (8e-7 kappa^2 an axis)."""
+    h = (12.0 / n[0],) * 2
+    s = Solver(n, h, gamma=1.0, nu=1.05, g=0.0, omega=omega, dt=4 * kappa * h[0] ** 2)
+    for ax in (0, 1):
+        s.set_solver(ax, "hybrid")
+    s.init_analytic(1)
+    s.step_imag(2)
+    s.step_real(1)
+    n0 = s.observables()["norm"]
+    s.step_real(STEPS)
+    assert abs(s.observables()["norm"] - n0) < per_step * STEPS
